@@ -1,41 +1,29 @@
 // Gradient of the Stage I cost S(1) of a noise-free rollout with respect to
-// its T x 4 controls, by reverse mode (adjoint) through the rollout: the
-// dynamics' vector-Jacobian products at the stages of the classical RK4
-// step, the quaternion renormalisation, and the cost terms (tracking, velocity
-// norm, control, goal, collision).  Not a step of the paper: it serves the
-// gradient refinement of the updated nominals before Stage II.
+// its T x 4 controls, by reverse mode (adjoint) through the rollout.  Not a
+// step of the paper: it serves the gradient refinement of the updated nominals
+// before Stage II and the cost-and-gradient entry point.
 //
-// One warp per control sequence.  Every lane runs the same serial RK4 chain on
-// the same operands (so all lanes hold the same values); the nearest-point
-// queries and the state terms of each 8-step segment run side by side on the
-// lanes.  The forward pass keeps a checkpoint every 8 steps; the backward pass
-// recomputes each 8-step segment from its checkpoint.
+// Every recurrence over the steps is a scan, one step per lane (thread).
+// Forward: rollout_by_scans' prefix products and sums.  Backward, with
+// L_{k+1} = dS/dx_{k+1} (the state terms at x_{k+1} plus what flows back from
+// later steps):
+//   position  Lp_{k+1} = sum_{i >= k} gp_i
+//   velocity  Lv_{k+1} = sum_{i >= k} (gv_i + h Lp_{i+2})
+//   attitude  the step is q_{k+1} = q_k (x) m_k / |q_k (x) m_k|, m_k from u_k
+//     alone.  Its transposed Jacobian maps l to ((P l) / |y|) (x) conj(m_k), P
+//     the projection off q_{k+1} and |y| = |m_k| for a unit q_k.  Multiplied
+//     by conj(q_k) on the right this is (P l) (x) conj(q_{k+1}): the vector
+//     part of l (x) conj(q), the adjoint in world axes, passes through a step
+//     unchanged, and the scalar part is what P removes.  So
+//     tau_{k+1} = vec(Lq_{k+1} (x) conj(q_{k+1})) is a suffix sum too: of the
+//     attitude state terms and of what each step's translation contributes.
+// Then dS/du_k of every step in parallel.
 #pragma once
 
 #include "device.cuh"
 #include "internal.h"
 
 namespace aero {
-
-constexpr int kCkpt = 8;  // steps per checkpoint segment
-
-// Scratch of one warp in shared memory.
-struct AdjScratch {
-  float ck[(kMaxT / kCkpt + 1) * 10];  // checkpoints x_0, x_8, x_16, ...
-  float seg[(kCkpt + 1) * 10];         // the states of one segment
-  float gs[kCkpt][10];                 // state-term gradients of the segment's states
-  float d2[kCkpt];                     // their nearest-point squared distances
-  float4 nearest[kCkpt];               // and nearest points
-};
-
-__device__ __forceinline__ void state_store(float* d, const State& x) {
-#pragma unroll
-  for (int i = 0; i < 3; ++i) d[i] = x.p[i];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) d[3 + i] = x.q[i];
-#pragma unroll
-  for (int i = 0; i < 3; ++i) d[7 + i] = x.v[i];
-}
 
 __device__ __forceinline__ State state_load(const float* d) {
   State x;
@@ -46,50 +34,6 @@ __device__ __forceinline__ State state_load(const float* d) {
 #pragma unroll
   for (int i = 0; i < 3; ++i) x.v[i] = d[7 + i];
   return x;
-}
-
-// Nearest collision points of the n <= 8 states seg[1..n] by the warp, four
-// lanes per state: squared distances (d_max^2 when none is closer) and the
-// nearest points into sc.d2 / sc.nearest.  Among equidistant points the one of
-// lowest item index wins (the collision set's order, as the oracle breaks
-// ties), whatever the order of the entries in the cell's list.
-__device__ __forceinline__ void warp_nn_segment(AdjScratch& sc, int n, const GridView& g,
-                                                float dmax2, int lane) {
-  const int k = lane >> 2, q = lane & 3;
-  float best = dmax2;
-  int bitem = 0x7fffffff;
-  float4 bp = make_float4(0.f, 0.f, 0.f, 0.f);
-  if (k < n) {
-    const float* x = sc.seg + (k + 1) * 10;
-    const int2 r = cell_range(x[0], x[1], x[2], g);
-    for (int i = q; i < r.y; i += 4) {
-      const float4 p = grid_point(g, r.x + i);
-      const float d2 = dist2_to(p, x[0], x[1], x[2]);
-      const int item = point_item(p);
-      if (d2 < best || (d2 == best && d2 < dmax2 && item < bitem)) {
-        best = d2;
-        bitem = item;
-        bp = p;
-      }
-    }
-  }
-#pragma unroll
-  for (int o = 1; o < 4; o <<= 1) {
-    const float ob = __shfl_xor_sync(0xffffffffu, best, o);
-    const int oi = __shfl_xor_sync(0xffffffffu, bitem, o);
-    const float ox = __shfl_xor_sync(0xffffffffu, bp.x, o);
-    const float oy = __shfl_xor_sync(0xffffffffu, bp.y, o);
-    const float oz = __shfl_xor_sync(0xffffffffu, bp.z, o);
-    if (ob < best || (ob == best && oi < bitem)) {
-      best = ob;
-      bitem = oi;
-      bp = make_float4(ox, oy, oz, bp.w);
-    }
-  }
-  if (k < n && q == 0) {
-    sc.d2[k] = best;
-    sc.nearest[k] = bitem != 0x7fffffff ? bp : make_float4(0.f, 0.f, 0.f, 0.f);
-  }
 }
 
 // Stage I state terms at the post-step state x against guide sample (gx, gy,
@@ -154,273 +98,415 @@ __device__ __forceinline__ float state_terms(const State& x, float gx, float gy,
   return c;
 }
 
-// xd = f(x, u) of the quadrotor model (Eq. dynamics) at a stage state.
-__device__ __forceinline__ void dyn_f(const float* x, float4 u, const DynParams& dp, float* xd) {
-  const float qw = x[3], qx = x[4], qy = x[5], qz = x[6];
-  xd[0] = x[7]; xd[1] = x[8]; xd[2] = x[9];
-  xd[3] = 0.5f * (-qx * u.y - qy * u.z - qz * u.w);
-  xd[4] = 0.5f * (qw * u.y + qy * u.w - qz * u.z);
-  xd[5] = 0.5f * (qw * u.z - qx * u.w + qz * u.y);
-  xd[6] = 0.5f * (qw * u.w + qx * u.z - qy * u.y);
-  float rx, ry, rz;
-  r_e3(qw, qx, qy, qz, rx, ry, rz);
-  const float f = u.x * dp.inv_mass;
-  xd[7] = f * rx; xd[8] = f * ry; xd[9] = f * rz - dp.g;
+// One step's adjoint: from the start attitude q, the control u and the adjoints
+// lp, lv of the step's end position and velocity, the parts that do not need
+// the end attitude's adjoint; step_adjoint_controls adds that one.  With
+// a = q (x) [0, w/2], hh = h^2 |w|^2 / 4 and the RK4 stage attitudes q_i =
+// alpha_i q + beta_i a of the closed-form step (see rk4_step), the position and
+// velocity increments are sums of r(q_i) = R(q_i) e3 / 2, so the adjoint of q_i
+// is r'(q_i)^T w_i with w_1 = Wp + Wv, w_2 = w_3 = Wp + 2 Wv, w_4 = Wv (Wp, Wv: lp
+// and lv times the increments' factors): four 4-vectors instead of a reverse
+// sweep over the four stage states.
+struct StepAdjoint {
+  float ga[4];  // adjoint of a
+  float ghh;    // adjoint of hh
+  float gF;     // adjoint of the thrust
+};
+
+// r'(q)^T w, r(q) = (xz + wy, yz - wx, 1/2 - x^2 - y^2).
+__device__ __forceinline__ void r_vjp(const float* q, const float* w, float* g) {
+  g[0] = w[0] * q[2] - w[1] * q[1];
+  g[1] = w[0] * q[3] - w[1] * q[0] - 2.0f * w[2] * q[1];
+  g[2] = w[0] * q[0] + w[1] * q[3] - 2.0f * w[2] * q[2];
+  g[3] = w[0] * q[1] + w[1] * q[2];
 }
 
-// w^T df/dx added to gx, w^T df/du added to gu, at stage state x.
-__device__ __forceinline__ void dyn_vjp(const float* x, float4 u, const DynParams& dp,
-                                        const float* w, float* gx, float* gu) {
-  const float qw = x[3], qx = x[4], qy = x[5], qz = x[6];
-  const float ox = u.y, oy = u.z, oz = u.w;
-  gx[7] += w[0]; gx[8] += w[1]; gx[9] += w[2];
-  const float W0 = 0.5f * w[3], W1 = 0.5f * w[4], W2 = 0.5f * w[5], W3 = 0.5f * w[6];
-  gx[3] += W1 * ox + W2 * oy + W3 * oz;
-  gx[4] += -W0 * ox - W2 * oz + W3 * oy;
-  gx[5] += -W0 * oy + W1 * oz - W3 * ox;
-  gx[6] += -W0 * oz - W1 * oy + W2 * ox;
-  gu[1] += -W0 * qx + W1 * qw + W2 * qz - W3 * qy;
-  gu[2] += -W0 * qy - W1 * qz + W2 * qw + W3 * qx;
-  gu[3] += -W0 * qz + W1 * qy - W2 * qx + W3 * qw;
-  const float V0 = w[7], V1 = w[8], V2 = w[9];
-  float rx, ry, rz;
-  r_e3(qw, qx, qy, qz, rx, ry, rz);
-  gu[0] += (V0 * rx + V1 * ry + V2 * rz) * dp.inv_mass;
-  const float s = u.x * dp.inv_mass;
-  gx[3] += s * (2.0f * qy * V0 - 2.0f * qx * V1);
-  gx[4] += s * (2.0f * qz * V0 - 2.0f * qw * V1 - 4.0f * qx * V2);
-  gx[5] += s * (2.0f * qw * V0 + 2.0f * qz * V1 - 4.0f * qy * V2);
-  gx[6] += s * (2.0f * qx * V0 + 2.0f * qy * V1);
+__device__ __forceinline__ float dot4(const float* a, const float* b) {
+  return a[0] * b[0] + a[1] * b[1] + a[2] * b[2] + a[3] * b[3];
 }
 
-// The stage states of one RK4 step from x with control u (Eq. dynamics):
-// t2 = x + h/2 k1, t3 = x + h/2 k2, t4 = x + h k3, and the quaternion before
-// renormalisation y = q + h/6 (k1 + 2 k2 + 2 k3 + k4) (quaternion part).
-__device__ __forceinline__ void rk4_stages(const float* x, float4 u, const DynParams& dp, float* t2,
-                                           float* t3, float* t4, float* y) {
+// a = q (x) [0, w/2] and hh of a step.
+__device__ __forceinline__ float step_a(const float* q, float4 u, float h, float* a) {
+  const float hx = 0.5f * u.y, hy = 0.5f * u.z, hz = 0.5f * u.w;
+  a[0] = -q[1] * hx - q[2] * hy - q[3] * hz;
+  a[1] = q[0] * hx + q[2] * hz - q[3] * hy;
+  a[2] = q[0] * hy - q[1] * hz + q[3] * hx;
+  a[3] = q[0] * hz + q[1] * hy - q[2] * hx;
+  return h * h * (hx * hx + hy * hy + hz * hz);
+}
+
+// Vector part of l (x) conj(q).
+__device__ __forceinline__ float3 vec_mul_conj(const float* l, const float* q) {
+  return make_float3(-l[0] * q[1] + l[1] * q[0] - l[2] * q[3] + l[3] * q[2],
+                     -l[0] * q[2] + l[1] * q[3] + l[2] * q[0] - l[3] * q[1],
+                     -l[0] * q[3] - l[1] * q[2] + l[2] * q[1] + l[3] * q[0]);
+}
+
+// The translation's part of the step's adjoint into s; returns what it adds to
+// tau of the step's start state.
+__device__ __forceinline__ float3 step_adjoint_translation(const float* q, float4 u, const DynParams& dp,
+                                                           float3 lp, float3 lv, StepAdjoint& s) {
   const float h = dp.dt;
-  float k1[10], k2[10], k3[10], k4[10];
-  dyn_f(x, u, dp, k1);
+  float a[4];
+  const float hh = step_a(q, u, h, a);
+  const float c3 = 1.0f - 0.25f * hh, c4 = 1.0f - 0.5f * hh, hb = 0.5f * h, h4 = h * c3;
+  float q2[4], q3[4], q4[4];
 #pragma unroll
-  for (int i = 0; i < 10; ++i) t2[i] = x[i] + 0.5f * h * k1[i];
-  dyn_f(t2, u, dp, k2);
-#pragma unroll
-  for (int i = 0; i < 10; ++i) t3[i] = x[i] + 0.5f * h * k2[i];
-  dyn_f(t3, u, dp, k3);
-#pragma unroll
-  for (int i = 0; i < 10; ++i) t4[i] = x[i] + h * k3[i];
-  dyn_f(t4, u, dp, k4);
-#pragma unroll
-  for (int i = 0; i < 4; ++i)
-    y[i] = x[3 + i] + h * (1.0f / 6.0f) * (k1[3 + i] + 2.0f * k2[3 + i] + 2.0f * k3[3 + i] + k4[3 + i]);
-}
-
-// Reverse of one RK4 step given its stage states: lam holds dS/dx_{j+1} on
-// entry and dS/dx_j on return; gu gets dS/du_j from the dynamics.  Through the
-// renormalisation q+ = y/|y| (projection (I - q+ q+^T)/|y|), then the four
-// stages in reverse.
-__device__ __forceinline__ void rk4_vjp_stages(const float* x, const float* t2, const float* t3,
-                                               const float* t4, const float* y, float4 u,
-                                               const DynParams& dp, float* lam, float* gu) {
-  const float h = dp.dt;
-  const float inv = rsqrtf(y[0] * y[0] + y[1] * y[1] + y[2] * y[2] + y[3] * y[3]);
-  const float dot = (y[0] * lam[3] + y[1] * lam[4] + y[2] * lam[5] + y[3] * lam[6]) * inv;
-  float ly[10];
-#pragma unroll
-  for (int i = 0; i < 10; ++i) ly[i] = lam[i];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) ly[3 + i] = (lam[3 + i] - y[i] * inv * dot) * inv;
-  float l1[10], l2[10], l3[10], l4[10], lt[10];
-#pragma unroll
-  for (int i = 0; i < 10; ++i) {
-    lam[i] = ly[i];
-    l1[i] = h * (1.0f / 6.0f) * ly[i];
-    l2[i] = h * (1.0f / 3.0f) * ly[i];
-    l3[i] = l2[i];
-    l4[i] = l1[i];
+  for (int i = 0; i < 4; ++i) {
+    q2[i] = q[i] + hb * a[i];
+    q3[i] = c3 * q[i] + hb * a[i];
+    q4[i] = c4 * q[i] + h4 * a[i];
   }
+  const float kp = h * h * (1.0f / 3.0f) * dp.inv_mass, kv = h * (1.0f / 3.0f) * dp.inv_mass;
+  const float P[3] = {kp * lp.x, kp * lp.y, kp * lp.z}, V[3] = {kv * lv.x, kv * lv.y, kv * lv.z};
+  float w1[3], w2[3];
 #pragma unroll
-  for (int i = 0; i < 10; ++i) lt[i] = 0.0f;
-  dyn_vjp(t4, u, dp, l4, lt, gu);
+  for (int i = 0; i < 3; ++i) {
+    w1[i] = P[i] + V[i];
+    w2[i] = w1[i] + V[i];
+  }
+  // the thrust's adjoint: w_i . r(q_i) summed (the factors hold 1/m, not F/m)
+  auto r_dot = [](const float* w, const float* z) {
+    float rx, ry, rz;
+    r_e3_half(z[0], z[1], z[2], z[3], rx, ry, rz);
+    return w[0] * rx + w[1] * ry + w[2] * rz;
+  };
+  s.gF = r_dot(w1, q) + r_dot(w2, q2) + r_dot(w2, q3) + r_dot(V, q4);
+  float g1[4], g2[4], g3[4], g4[4], gq[4];
+  r_vjp(q, w1, g1);
+  r_vjp(q2, w2, g2);
+  r_vjp(q3, w2, g3);
+  r_vjp(q4, V, g4);
 #pragma unroll
-  for (int i = 0; i < 10; ++i) { lam[i] += lt[i]; l3[i] += h * lt[i]; lt[i] = 0.0f; }
-  dyn_vjp(t3, u, dp, l3, lt, gu);
+  for (int i = 0; i < 4; ++i) {
+    g1[i] *= u.x;
+    g2[i] *= u.x;
+    g3[i] *= u.x;
+    g4[i] *= u.x;
+    s.ga[i] = hb * (g2[i] + g3[i]) + h4 * g4[i];
+    gq[i] = g1[i] + g2[i] + c3 * g3[i] + c4 * g4[i];
+  }
+  s.ghh = -0.25f * (dot4(g3, q) + h * dot4(g4, a)) - 0.5f * dot4(g4, q);
+  // through a = q (x) [0, w/2]: ga (x) [0, -w/2]
+  float at[4];
+  step_a(s.ga, make_float4(0.f, -u.y, -u.z, -u.w), h, at);
 #pragma unroll
-  for (int i = 0; i < 10; ++i) { lam[i] += lt[i]; l2[i] += 0.5f * h * lt[i]; lt[i] = 0.0f; }
-  dyn_vjp(t2, u, dp, l2, lt, gu);
-#pragma unroll
-  for (int i = 0; i < 10; ++i) { lam[i] += lt[i]; l1[i] += 0.5f * h * lt[i]; }
-  dyn_vjp(x, u, dp, l1, lam, gu);
+  for (int i = 0; i < 4; ++i) gq[i] += at[i];
+  return vec_mul_conj(gq, q);
 }
 
-// Reverse of one RK4 step from x with control u (stage states recomputed).
-__device__ __forceinline__ void rk4_vjp(const float* x, float4 u, const DynParams& dp, float* lam,
-                                        float* gu) {
-  float t2[10], t3[10], t4[10], y[4];
-  rk4_stages(x, u, dp, t2, t3, t4, y);
-  rk4_vjp_stages(x, t2, t3, t4, y, u, dp, lam, gu);
+// dS/du of the step from the translation's part s and tau of its end state.
+__device__ __forceinline__ float4 step_adjoint_controls(const float* q, float4 u, const DynParams& dp,
+                                                        const StepAdjoint& s, float3 tau) {
+  const float h = dp.dt;
+  float a[4], y[4];
+  const float hh = step_a(q, u, h, a);
+  const float cq = 1.0f - 0.5f * hh + hh * hh * (1.0f / 24.0f);
+  const float ca = h * (1.0f - hh * (1.0f / 6.0f));
+#pragma unroll
+  for (int i = 0; i < 4; ++i) y[i] = cq * q[i] + ca * a[i];
+  // the adjoint of y: (tau (x) q_{k+1}) / |y|, q_{k+1} = y / |y|
+  const float inv2 = __frcp_rn(dot4(y, y));
+  const float tx = tau.x * inv2, ty = tau.y * inv2, tz = tau.z * inv2;
+  const float l[4] = {-tx * y[1] - ty * y[2] - tz * y[3], tx * y[0] + ty * y[3] - tz * y[2],
+                      -tx * y[3] + ty * y[0] + tz * y[1], tx * y[2] - ty * y[1] + tz * y[0]};
+  const float ghh = s.ghh + (hh * (1.0f / 12.0f) - 0.5f) * dot4(l, q) - h * (1.0f / 6.0f) * dot4(l, a);
+  float g[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) g[i] = s.ga[i] + ca * l[i];
+  // w_c = 2 (w/2)_c; hh = h^2 |w/2|^2
+  const float k = 0.5f * h * h * ghh;
+  return make_float4(s.gF,
+                     0.5f * (-g[0] * q[1] + g[1] * q[0] + g[2] * q[3] - g[3] * q[2]) + k * u.y,
+                     0.5f * (-g[0] * q[2] - g[1] * q[3] + g[2] * q[0] + g[3] * q[1]) + k * u.z,
+                     0.5f * (-g[0] * q[3] + g[1] * q[2] - g[2] * q[1] + g[3] * q[0]) + k * u.w);
 }
 
-// S(1) of the noise-free rollout of u (shared, T entries) from x0 and, with
-// kGrad, dS/du into g (shared, T entries).  guide: T x 3 (shared or global).
-// Called by all 32 lanes of one warp; returns S on every lane.
+// The control terms' part of dS/du_t added to a: Q_c |u_t|^2 (t <= T-2) and
+// Q_cd |u_t - u_{t-1}|^2 (1 <= t <= T-2).
+__device__ __forceinline__ float4 control_terms_grad(float4 a, const float4* u, int t, int T,
+                                                     const CostParams& cp) {
+  const float4 ut = u[t];
+  if (t <= T - 2) {
+    a.x += 2.0f * cp.Q_c * ut.x; a.y += 2.0f * cp.Q_c * ut.y;
+    a.z += 2.0f * cp.Q_c * ut.z; a.w += 2.0f * cp.Q_c * ut.w;
+  }
+  if (t >= 1 && t <= T - 2) {
+    const float4 b = u[t - 1];
+    a.x += 2.0f * cp.Q_cd * (ut.x - b.x); a.y += 2.0f * cp.Q_cd * (ut.y - b.y);
+    a.z += 2.0f * cp.Q_cd * (ut.z - b.z); a.w += 2.0f * cp.Q_cd * (ut.w - b.w);
+  }
+  if (t + 1 <= T - 2) {
+    const float4 c = u[t + 1];
+    a.x -= 2.0f * cp.Q_cd * (c.x - ut.x); a.y -= 2.0f * cp.Q_cd * (c.y - ut.y);
+    a.z -= 2.0f * cp.Q_cd * (c.z - ut.z); a.w -= 2.0f * cp.Q_cd * (c.w - ut.w);
+  }
+  return a;
+}
+
+// ---------------------------------------------------------------------------
+// Cost and gradient of one sequence by one warp.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ float3 add3(float3 a, float3 b) {
+  return make_float3(a.x + b.x, a.y + b.y, a.z + b.z);
+}
+
+__device__ __forceinline__ float3 shfl3(float3 v, int src) {
+  return make_float3(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src),
+                     __shfl_sync(0xffffffffu, v.z, src));
+}
+
+// Inclusive sums over the lanes up to this one (kUp) or from this one on.
+template <bool kUp>
+__device__ __forceinline__ float3 warp_scan3(float3 x, int lane) {
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const float a = kUp ? __shfl_up_sync(0xffffffffu, x.x, o) : __shfl_down_sync(0xffffffffu, x.x, o);
+    const float b = kUp ? __shfl_up_sync(0xffffffffu, x.y, o) : __shfl_down_sync(0xffffffffu, x.y, o);
+    const float c = kUp ? __shfl_up_sync(0xffffffffu, x.z, o) : __shfl_down_sync(0xffffffffu, x.z, o);
+    if (kUp ? lane >= o : lane + o < 32) x = make_float3(x.x + a, x.y + b, x.z + c);
+  }
+  return x;
+}
+
+// The value of the lane before (kUp) or after this one; `edge` at the end.
+template <bool kUp>
+__device__ __forceinline__ float3 warp_next3(float3 x, float3 edge, int lane) {
+  const float a = kUp ? __shfl_up_sync(0xffffffffu, x.x, 1) : __shfl_down_sync(0xffffffffu, x.x, 1);
+  const float b = kUp ? __shfl_up_sync(0xffffffffu, x.y, 1) : __shfl_down_sync(0xffffffffu, x.y, 1);
+  const float c = kUp ? __shfl_up_sync(0xffffffffu, x.z, 1) : __shfl_down_sync(0xffffffffu, x.z, 1);
+  return lane == (kUp ? 0 : 31) ? edge : make_float3(a, b, c);
+}
+
+// Nearest collision point of every lane's query (all 32 lanes call it): the
+// squared distance into d2 (d_max^2 when none is closer) and the point.  Lists
+// of at most kOwnList entries are scanned by their own lane, longer ones by the
+// whole warp in turn.  Among equidistant points the one of lowest item index
+// wins (the collision set's order, as the oracle breaks ties), whatever the
+// order of the entries in the cell's list.
+constexpr int kOwnList = 8;
+
+__device__ __forceinline__ void warp_nearest(const GridView& g, int2 r, float px, float py, float pz,
+                                             float dmax2, int lane, float& d2_out, float4& near) {
+  float best = dmax2;
+  int bitem = 0x7fffffff;
+  float4 bp = make_float4(0.f, 0.f, 0.f, 0.f);
+  auto visit = [&](int e, float qx, float qy, float qz) {
+    const float4 p = grid_point(g, e);
+    const float d2 = dist2_to(p, qx, qy, qz);
+    const int item = point_item(p);
+    if (d2 < best || (d2 == best && d2 < dmax2 && item < bitem)) {
+      best = d2;
+      bitem = item;
+      bp = p;
+    }
+  };
+  const bool lng = r.y > kOwnList;
+  unsigned pend = __ballot_sync(0xffffffffu, lng);
+  while (pend) {
+    const int L = __ffs(pend) - 1;
+    pend &= pend - 1;
+    const int first = __shfl_sync(0xffffffffu, r.x, L), n = __shfl_sync(0xffffffffu, r.y, L);
+    const float qx = __shfl_sync(0xffffffffu, px, L), qy = __shfl_sync(0xffffffffu, py, L),
+                qz = __shfl_sync(0xffffffffu, pz, L);
+    // the lanes' own results wait in registers while they work for lane L
+    const float kb = best;
+    const int ki = bitem;
+    const float4 kp = bp;
+    best = dmax2;
+    bitem = 0x7fffffff;
+    bp = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = lane; i < n; i += 32) visit(first + i, qx, qy, qz);
+    const unsigned bits = __float_as_uint(best);  // non-negative: ordered as its bits
+    const unsigned m = __reduce_min_sync(0xffffffffu, bits);
+    const unsigned mi = __reduce_min_sync(0xffffffffu, bits == m ? (unsigned)bitem : 0x7fffffffu);
+    const int src = __ffs(__ballot_sync(0xffffffffu, bits == m && (unsigned)bitem == mi)) - 1;
+    const float4 p = make_float4(__shfl_sync(0xffffffffu, bp.x, src), __shfl_sync(0xffffffffu, bp.y, src),
+                                 __shfl_sync(0xffffffffu, bp.z, src), 0.f);
+    best = lane == L ? __uint_as_float(m) : kb;
+    bitem = lane == L ? (int)mi : ki;
+    bp = lane == L ? p : kp;
+  }
+  if (!lng)
+    for (int i = 0; i < r.y; ++i) visit(r.x + i, px, py, pz);
+  d2_out = best;
+  near = bp;
+}
+
+// Scratch of one warp in shared memory (floats), for horizon T: the controls T x 4,
+// the attitudes q_0 .. q_T and, per step, the state-term gradients gp, gv
+// and the attitude terms' part of tau.
+__host__ __device__ constexpr size_t cost_grad_words(int T) { return 4 * (size_t)T + 4 * (size_t)(T + 1) + 9 * (size_t)T + 3 & ~(size_t)3; }
+
+// S(1) of the noise-free rollout of U (global, T entries) from x0 and, with
+// kGrad, dS/dU into G (global).  guide: T x 3 (global).  Called by all 32 lanes
+// of one warp; returns S on every lane.
 //
-// Per 8-step segment: the serial RK4 steps (every lane, identical), the
-// segment's nearest-point queries side by side (four lanes per state), its
-// state terms side by side (one lane per state).  The backward pass
-// recomputes the segment from its checkpoint and runs only the serial
-// vector-Jacobian products in order.
+// 32 steps at a time, one per lane: the scans above with the last lane's
+// state (forward) or the first lane's adjoints (backward) carried to the
+// next 32.  A sequence of 40 steps with its gradient takes two rounds each way
+// instead of 40 dependent RK4 steps forward and 40 again with their reverse
+// sweeps backward, which every lane computed alike: 2048 such sequences
+// 90.7 -> 14.8 us (bound by the latency of the scans' shuffles and of the
+// candidate lists).
 template <bool kGrad>
-__device__ float warp_cost_grad(const float4* u, float4* g, const float* guide, int T,
-                                const float* x0, const DynParams& dp, const CostParams& cp,
-                                const GridView& grid, AdjScratch& sc, int lane) {
+__device__ float warp_cost_grad(const float4* __restrict__ U, float4* __restrict__ G, const float* guide,
+                                int T, const float* x0, const DynParams& dp, const CostParams& cp,
+                                const GridView& grid, float* scratch, int lane) {
   const float dmax2 = cp.d_max * cp.d_max;
-  const int nseg = (T + kCkpt - 1) / kCkpt;
-  State x = state_load(x0);
+  const float h = dp.dt;
+  float4* const su = reinterpret_cast<float4*>(scratch);
+  float4* const sq = su + T;
+  float* const sg = reinterpret_cast<float*>(sq + T + 1);  // [9][T]
+  for (int t = lane; t < T; t += 32) su[t] = __ldg(U + t);
+  float4 qc = make_float4(x0[3], x0[4], x0[5], x0[6]);  // the round's first state
+  float3 pc = make_float3(x0[0], x0[1], x0[2]), vc = make_float3(x0[7], x0[8], x0[9]);
+  if (kGrad && lane == 0) sq[0] = qc;
+  __syncwarp();
+  const int rounds = (T + 31) / 32;
   float S = 0.0f;
-  for (int s = 0; s < nseg; ++s) {
-    const int j0 = s * kCkpt, n = min(T, j0 + kCkpt) - j0;
-    if (lane == 0) {
-      state_store(sc.ck + s * 10, x);
-      state_store(sc.seg, x);
+  for (int r = 0; r < rounds; ++r) {
+    const int j = 32 * r + lane;
+    const bool on = j < T;
+    const float4 u = on ? su[j] : make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 m = on ? rk4_attitude_coefs(u, dp) : make_float4(1.f, 0.f, 0.f, 0.f);
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const float4 y = shfl_up4(m, o);
+      if (lane >= o) m = quat_mul4(y, m);
     }
-    for (int k = 0; k < n; ++k) {
-      rk4_step(x, u[j0 + k], dp);
-      if (lane == 0) state_store(sc.seg + (k + 1) * 10, x);
+    float4 q1 = quat_mul4(qc, m);
+    const float inv = rsqrtf(q1.x * q1.x + q1.y * q1.y + q1.z * q1.z + q1.w * q1.w);
+    q1 = make_float4(q1.x * inv, q1.y * inv, q1.z * inv, q1.w * inv);
+    float4 q = shfl_up4(q1, 1);
+    if (lane == 0) q = qc;
+    const float qj[4] = {q.x, q.y, q.z, q.w};
+    float inc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    if (on) rk4_translation_increments(qj, u, dp, inc);
+    const float3 v1 = add3(vc, warp_scan3<true>(make_float3(inc[3], inc[4], inc[5]), lane));
+    const float3 vj = warp_next3<true>(v1, vc, lane);
+    const float3 p1 = add3(pc, warp_scan3<true>(make_float3(h * vj.x + inc[0], h * vj.y + inc[1],
+                                                            h * vj.z + inc[2]), lane));
+    float d2;
+    float4 near;
+    warp_nearest(grid, on ? cell_range(p1.x, p1.y, p1.z, grid) : make_int2(0, 0), p1.x, p1.y, p1.z,
+                 dmax2, lane, d2, near);
+    if (on) {
+      State x;
+      x.p[0] = p1.x; x.p[1] = p1.y; x.p[2] = p1.z;
+      x.q[0] = q1.x; x.q[1] = q1.y; x.q[2] = q1.z; x.q[3] = q1.w;
+      x.v[0] = v1.x; x.v[1] = v1.y; x.v[2] = v1.z;
+      float gs[10];
+      S += state_terms<kGrad>(x, guide[3 * j], guide[3 * j + 1], guide[3 * j + 2], d2, near, cp, dmax2, gs);
+      if (kGrad) {
+        sq[j + 1] = q1;
+        const float3 t = vec_mul_conj(gs + 3, x.q);
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+          sg[i * T + j] = gs[i];
+          sg[(3 + i) * T + j] = gs[7 + i];
+        }
+        sg[6 * T + j] = t.x;
+        sg[7 * T + j] = t.y;
+        sg[8 * T + j] = t.z;
+      }
+      // J_ctrl: Q_c |u_j|^2 (j <= T-2) and Q_cd |u_j - u_{j-1}|^2 (1 <= j <= T-2)
+      if (j <= T - 2) {
+        S += cp.Q_c * (u.x * u.x + u.y * u.y + u.z * u.z + u.w * u.w);
+        if (j >= 1) {
+          const float4 b = su[j - 1];
+          const float dx = u.x - b.x, dy = u.y - b.y, dz = u.z - b.z, dw = u.w - b.w;
+          S += cp.Q_cd * (dx * dx + dy * dy + dz * dz + dw * dw);
+        }
+      }
     }
-    __syncwarp();
-    warp_nn_segment(sc, n, grid, dmax2, lane);
-    __syncwarp();
-    float c = 0.0f;
-    if (lane < n) {
-      const int j = j0 + lane;
-      c = state_terms<false>(state_load(sc.seg + (lane + 1) * 10), guide[3 * j], guide[3 * j + 1],
-                             guide[3 * j + 2], sc.d2[lane], sc.nearest[lane], cp, dmax2, nullptr);
+    if (r + 1 < rounds) {
+      qc = make_float4(__shfl_sync(0xffffffffu, q1.x, 31), __shfl_sync(0xffffffffu, q1.y, 31),
+                       __shfl_sync(0xffffffffu, q1.z, 31), __shfl_sync(0xffffffffu, q1.w, 31));
+      vc = shfl3(v1, 31);
+      pc = shfl3(p1, 31);
     }
-    S += warp_sum(c);
-    __syncwarp();
   }
-  // J_ctrl: Q_c |u_t|^2 (t <= T-2) and Q_cd |u_t - u_{t-1}|^2 (1 <= t <= T-2)
-  float jc = 0.0f;
-  for (int t = lane; t <= T - 2; t += 32) {
-    const float4 a = u[t];
-    jc += cp.Q_c * (a.x * a.x + a.y * a.y + a.z * a.z + a.w * a.w);
-    if (t >= 1) {
-      const float4 b = u[t - 1];
-      const float dx = a.x - b.x, dy = a.y - b.y, dz = a.z - b.z, dw = a.w - b.w;
-      jc += cp.Q_cd * (dx * dx + dy * dy + dz * dz + dw * dw);
-    }
-  }
-  S += warp_sum(jc);
+  S = warp_sum(S);
   if constexpr (kGrad) {
-    float lam[10];
-#pragma unroll
-    for (int i = 0; i < 10; ++i) lam[i] = 0.0f;
-    for (int s = nseg - 1; s >= 0; --s) {
-      const int j0 = s * kCkpt, n = min(T, j0 + kCkpt) - j0;
-      // recompute the segment's states from its checkpoint
-      State y = state_load(sc.ck + s * 10);
-      if (lane == 0) state_store(sc.seg, y);
-      for (int k = 0; k < n; ++k) {
-        rk4_step(y, u[j0 + k], dp);
-        if (lane == 0) state_store(sc.seg + (k + 1) * 10, y);
-      }
-      __syncwarp();
-      warp_nn_segment(sc, n, grid, dmax2, lane);
-      __syncwarp();
-      if (lane < n) {
-        const int j = j0 + lane;
-        float gs[10];
-        state_terms<true>(state_load(sc.seg + (lane + 1) * 10), guide[3 * j], guide[3 * j + 1],
-                          guide[3 * j + 2], sc.d2[lane], sc.nearest[lane], cp, dmax2, gs);
-#pragma unroll
-        for (int i = 0; i < 10; ++i) sc.gs[lane][i] = gs[i];
-      }
-      __syncwarp();
-      for (int k = n - 1; k >= 0; --k) {
-#pragma unroll
-        for (int i = 0; i < 10; ++i) lam[i] += sc.gs[k][i];
-        float gu[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-        rk4_vjp(sc.seg + k * 10, u[j0 + k], dp, lam, gu);
-        if (lane == 0) g[j0 + k] = make_float4(gu[0], gu[1], gu[2], gu[3]);
-      }
-      __syncwarp();
-    }
-    // control terms
-    for (int t = lane; t < T; t += 32) {
-      float4 a = g[t];
-      const float4 ut = u[t];
-      if (t <= T - 2) {
-        a.x += 2.0f * cp.Q_c * ut.x; a.y += 2.0f * cp.Q_c * ut.y;
-        a.z += 2.0f * cp.Q_c * ut.z; a.w += 2.0f * cp.Q_c * ut.w;
-      }
-      if (t >= 1 && t <= T - 2) {
-        const float4 b = u[t - 1];
-        a.x += 2.0f * cp.Q_cd * (ut.x - b.x); a.y += 2.0f * cp.Q_cd * (ut.y - b.y);
-        a.z += 2.0f * cp.Q_cd * (ut.z - b.z); a.w += 2.0f * cp.Q_cd * (ut.w - b.w);
-      }
-      if (t + 1 >= 1 && t + 1 <= T - 2) {
-        const float4 c = u[t + 1];
-        a.x -= 2.0f * cp.Q_cd * (c.x - ut.x); a.y -= 2.0f * cp.Q_cd * (c.y - ut.y);
-        a.z -= 2.0f * cp.Q_cd * (c.z - ut.z); a.w -= 2.0f * cp.Q_cd * (c.w - ut.w);
-      }
-      g[t] = a;
-    }
     __syncwarp();
+    const float3 zero = make_float3(0.f, 0.f, 0.f);
+    float3 cp_p = zero, cp_v = zero, cp_t = zero;  // the later rounds' sums
+    for (int r = rounds - 1; r >= 0; --r) {
+      const int k = 32 * r + lane;
+      const bool on = k < T;
+      float3 gp = zero, gv = zero, tg = zero;
+      float4 u = make_float4(0.f, 0.f, 0.f, 0.f), q4 = make_float4(1.f, 0.f, 0.f, 0.f);
+      if (on) {
+        gp = make_float3(sg[k], sg[T + k], sg[2 * T + k]);
+        gv = make_float3(sg[3 * T + k], sg[4 * T + k], sg[5 * T + k]);
+        tg = make_float3(sg[6 * T + k], sg[7 * T + k], sg[8 * T + k]);
+        u = su[k];
+        q4 = sq[k];
+      }
+      const float q[4] = {q4.x, q4.y, q4.z, q4.w};
+      const float3 lp = add3(warp_scan3<false>(gp, lane), cp_p);  // Lp_{k+1}
+      const float3 lp2 = warp_next3<false>(lp, cp_p, lane);       // Lp_{k+2}
+      const float3 lv = add3(warp_scan3<false>(make_float3(gv.x + h * lp2.x, gv.y + h * lp2.y,
+                                                           gv.z + h * lp2.z), lane), cp_v);
+      StepAdjoint sa;
+      float3 bt = step_adjoint_translation(q, u, dp, lp, lv, sa);
+      if (!on) bt = zero;
+      const float3 ts = add3(warp_scan3<false>(add3(tg, bt), lane), cp_t);  // tau_k without tg_{k-1}
+      const float3 tau = add3(warp_next3<false>(ts, cp_t, lane), tg);       // tau_{k+1}
+      if (on) G[k] = control_terms_grad(step_adjoint_controls(q, u, dp, sa, tau), su, k, T, cp);
+      if (r > 0) {
+        cp_p = shfl3(lp, 0);
+        cp_v = shfl3(lv, 0);
+        cp_t = shfl3(ts, 0);
+      }
+    }
   }
   return S;
 }
 
 // ---------------------------------------------------------------------------
-// Gradient refinement by a whole CTA (the update kernels): the forward
-// states by scans over the steps (rollout_by_scans); the backward pass split
-// by dependence (suffix sums for the position and velocity adjoints, the 4x4
-// attitude recurrence on one thread, the vector-Jacobian products of every
-// step in parallel); everything else over the CTA: the stage states of every
-// step, the nearest point of every
-// state (candidate lists cut into items of kRefItem entries; a 64-bit atomic
-// minimum of (squared distance bits, item index) keeps the lowest item among
-// equidistant points, the collision set's order), the state terms and their
-// gradients, the control terms and the clamped step.  The same arithmetic as
-// warp_cost_grad<true> followed by the clamped step.
+// Gradient refinement by a whole CTA (the update kernels), one step per
+// thread: the forward states by scans over the steps (rollout_by_scans), the
+// nearest point of every state (candidate lists cut into items of kRefItem
+// entries; a 64-bit atomic minimum of (squared distance bits, item index) keeps
+// the lowest item among equidistant points, the collision set's order), the
+// state terms and their gradients, three suffix sums for the adjoints, the
+// control terms and the clamped step.  Latency bound (one CTA per instance, the
+// barriers of the scans in a chain): five steps added 30 us to a planning step
+// of E = 8, K = 1024, T = 40 with the attitude adjoint as a scan of 4x4 affine
+// maps and the stages' reverse sweep twice, 20 us with the sums.
 // ---------------------------------------------------------------------------
 constexpr int kRefItem = 8;
 
 struct RefineScratch {
   float4* tot;               // warps: scan totals of the forward rollout
-  float4* g;                 // T: dS/du
   unsigned long long* key;   // T: (bits(d2) << 32) | item of the nearest point of x_{j+1}
   float4* near;              // T: that point (entries holding points: found by a second pass)
   int2* qrange;              // T: candidate range of each listed query
   int2* scan;                // warps: block-scan totals
   float* xs;                 // (T + 1) x 10: states x_0 .. x_T
-  float* st;                 // T x 34: stage states t2, t3, t4 and y of step j
-  float* gs;                 // T x 10: state-term gradients at x_{j+1}
+  float* gs;                 // T x 9: state-term gradients at x_{j+1} (gp, gv, part of tau)
   int* qitem;                // T + 1: first item of each listed query
   int* qslot;                // T: step of each listed query
-  float* afm;                // 4 x 20: the attitude adjoint scan's warp compositions
 };
 
 __host__ __device__ constexpr size_t refine_smem_bytes(int T, int warps) {
-  return 16 * (size_t)warps + 16 * (size_t)T + 8 * (size_t)T + 16 * (size_t)T + 8 * (size_t)T + 8 * (size_t)warps +
-         4 * (size_t)(T + 1) * 10 + 4 * (size_t)T * 34 + 4 * (size_t)T * 10 + 4 * (size_t)(T + 1) +
-         4 * (size_t)T + 4 * 80;
+  return 16 * (size_t)warps + 8 * (size_t)T + 16 * (size_t)T + 8 * (size_t)T + 8 * (size_t)warps +
+         4 * (size_t)(T + 1) * 10 + 4 * (size_t)T * 9 + 4 * (size_t)(T + 1) + 4 * (size_t)T;
 }
 
 __device__ __forceinline__ RefineScratch refine_layout(unsigned char* base, int T, int warps) {
   RefineScratch r;
   r.tot = reinterpret_cast<float4*>(base);
-  r.g = r.tot + warps;
-  r.key = reinterpret_cast<unsigned long long*>(r.g + T);
-  r.near = reinterpret_cast<float4*>(r.key + T);
-  r.qrange = reinterpret_cast<int2*>(r.near + T);
+  r.near = r.tot + warps;
+  r.key = reinterpret_cast<unsigned long long*>(r.near + T);
+  r.qrange = reinterpret_cast<int2*>(r.key + T);
   r.scan = r.qrange + T;
   r.xs = reinterpret_cast<float*>(r.scan + warps);
-  r.st = r.xs + (size_t)(T + 1) * 10;
-  r.gs = r.st + (size_t)T * 34;
-  r.qitem = reinterpret_cast<int*>(r.gs + (size_t)T * 10);
+  r.gs = r.xs + (size_t)(T + 1) * 10;
+  r.qitem = reinterpret_cast<int*>(r.gs + (size_t)T * 9);
   r.qslot = r.qitem + T + 1;
-  r.afm = reinterpret_cast<float*>(r.qslot + T);
   return r;
 }
 
@@ -439,11 +525,9 @@ __device__ void block_refine(float4* u, const float* guide, int T, const float* 
   for (int r = 0; r < steps; ++r) {
     // forward: the states x_0 .. x_T, by scans over the steps
     rollout_by_scans<kThreads / 32>(u, T, x0, dp, rs.xs, rs.tot);
-    // step tid: its stage states and the candidate range of x_{tid+1}
+    // the candidate range of x_{tid+1}
     int2 rg = make_int2(0, 0);
     if (tid < T) {
-      float* stj = rs.st + (size_t)tid * 34;
-      rk4_stages(rs.xs + tid * 10, u[tid], dp, stj, stj + 10, stj + 20, stj + 30);
       rs.key[tid] = none;
       const float* x1 = rs.xs + (tid + 1) * 10;
       rg = cell_range(x1[0], x1[1], x1[2], grid);
@@ -512,194 +596,47 @@ __device__ void block_refine(float4* u, const float* guide, int T, const float* 
       const float4 nearest = bi == 0xffffffffu ? make_float4(0.f, 0.f, 0.f, 0.f)
                              : grid.cand       ? __ldg(grid.pts + bi)
                                                : rs.near[tid];
-      state_terms<true>(state_load(rs.xs + (tid + 1) * 10), guide[3 * tid], guide[3 * tid + 1],
-                        guide[3 * tid + 2], d2, nearest, cp, dmax2, rs.gs + tid * 10);
+      const State x1 = state_load(rs.xs + (tid + 1) * 10);
+      float gs[10];
+      state_terms<true>(x1, guide[3 * tid], guide[3 * tid + 1], guide[3 * tid + 2], d2, nearest, cp,
+                        dmax2, gs);
+      const float3 t = vec_mul_conj(gs + 3, x1.q);
+      float* g = rs.gs + tid * 9;
+      g[0] = gs[0]; g[1] = gs[1]; g[2] = gs[2];
+      g[3] = gs[7]; g[4] = gs[8]; g[5] = gs[9];
+      g[6] = t.x; g[7] = t.y; g[8] = t.z;
     }
     __syncthreads();
-    // backward.  With L_{k+1} = dS/dx_{k+1} (the state terms at x_{k+1} plus
-    // what flows back from later steps), L_{k+1} = gs[k] + J_{k+1}^T L_{k+2},
-    // J the step Jacobian.  Positions feed only positions and velocities only
-    // positions and velocities, so the position and velocity parts are
-    // suffix sums: Lp_{k+1} = sum_{i >= k} gs_p[i], Lv_{k+1} = sum_{i >= k}
-    // (gs_v[i] + h Lp_{i+2}).  The attitude part is the linear recurrence
-    // Lq_{k+1} = gs_q[k] + b_{k+1} + A_{k+1}^T Lq_{k+2}: b the attitude part of
-    // J^T (Lp, 0, Lv) (the step's vector-Jacobian product, in parallel), A the
-    // 4x4 attitude Jacobian, whose transpose is applied in closed form: the
-    // unnormalised y = q (x) m, so A^T l = ((l - yh (yh . l)) / |y|) (x) conj(m),
-    // yh = y / |y|; one thread chains it.  Then every step's dS/du_k is the
-    // control part of J_k^T L_{k+1}, in parallel.
-    {
-      const float h = dp.dt;
-      // (a) the suffix sums, thread t taking step k = T - 1 - t
-      const int k = T - 1 - tid;
-      const bool on = tid < T;
-      const float* g = rs.gs + (on ? k : 0) * 10;
-      const float3 gp = on ? make_float3(g[0], g[1], g[2]) : make_float3(0.f, 0.f, 0.f);
-      const float3 gv = on ? make_float3(g[7], g[8], g[9]) : make_float3(0.f, 0.f, 0.f);
-      const float3 lp = block_sum_scan3<kThreads / 32>(gp, rs.tot);
-      const float3 lp2 = make_float3(lp.x - gp.x, lp.y - gp.y, lp.z - gp.z);  // Lp_{k+2}
-      const float3 lv = block_sum_scan3<kThreads / 32>(
-          make_float3(gv.x + h * lp2.x, gv.y + h * lp2.y, gv.z + h * lp2.z), rs.tot);
-      if (on) {
-        float* L = rs.gs + k * 10;
-        L[0] = lp.x; L[1] = lp.y; L[2] = lp.z;
-        L[7] = lv.x; L[8] = lv.y; L[9] = lv.z;
-      }
-      __syncthreads();
-      // (b) b_k for every step k = tid, into rs.g
-      if (tid < T) {
-        const float* L = rs.gs + tid * 10;
-        float lam[10] = {L[0], L[1], L[2], 0.f, 0.f, 0.f, 0.f, L[7], L[8], L[9]};
-        float gu[4] = {0.f, 0.f, 0.f, 0.f};
-        const float* stk = rs.st + (size_t)tid * 34;
-        rk4_vjp_stages(rs.xs + tid * 10, stk, stk + 10, stk + 20, stk + 30, u[tid], dp, lam, gu);
-        rs.g[tid] = make_float4(lam[3], lam[4], lam[5], lam[6]);
-      }
-      __syncthreads();
-      // (c) the attitude recurrence Lq_k = C_k + A_{k+1}^T Lq_{k+1} (k = T-2
-      // .. 0; C_k = gs_q[k] + b_{k+1}; Lq_{T-1} = gs_q[T-1]) is affine in Lq:
-      // thread t = T-2-k holds the map x -> C_k + M x (M = A_{k+1}^T as a 4x4
-      // matrix, its columns the images of the unit vectors), and an inclusive
-      // scan composes the maps, later ones outside, so that thread t ends with
-      // the composition that takes Lq_{T-1} to Lq_k.  T - 1 <= 127 maps: up to
-      // four warps, each carrying the earlier warps' compositions.
-      static_assert(kMaxT - 1 <= 128 && kThreads >= 128, "the attitude adjoint scan spans four warps");
-      {
-        const int kk = T - 2 - tid, wid = tid >> 5;
-        const bool on = kk >= 0;
-        float M[16], c[4];
-#pragma unroll
-        for (int i = 0; i < 16; ++i) M[i] = (i % 5 == 0) ? 1.0f : 0.0f;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) c[i] = 0.0f;
-        if (on) {
-          const int j = kk + 1;  // A_j: the attitude Jacobian of step j
-          const float* y = rs.st + (size_t)j * 34 + 30;
-          const float inv = rsqrtf(y[0] * y[0] + y[1] * y[1] + y[2] * y[2] + y[3] * y[3]);
-          const float4 m = rk4_attitude_coefs(u[j], dp);
-          const float4 mc = make_float4(m.x, -m.y, -m.z, -m.w);
-#pragma unroll
-          for (int col = 0; col < 4; ++col) {
-            // A_j^T e_col = ((e_col - yh (yh . e_col)) / |y|) (x) conj(m)
-            const float d = y[col] * inv * inv;
-            const float4 pl = make_float4(((col == 0 ? 1.f : 0.f) - y[0] * d) * inv,
-                                          ((col == 1 ? 1.f : 0.f) - y[1] * d) * inv,
-                                          ((col == 2 ? 1.f : 0.f) - y[2] * d) * inv,
-                                          ((col == 3 ? 1.f : 0.f) - y[3] * d) * inv);
-            const float4 at = quat_mul4(pl, mc);
-            M[col] = at.x;
-            M[4 + col] = at.y;
-            M[8 + col] = at.z;
-            M[12 + col] = at.w;
-          }
-          const float* Lk = rs.gs + kk * 10 + 3;
-          const float4 b = rs.g[j];
-          c[0] = Lk[0] + b.x;
-          c[1] = Lk[1] + b.y;
-          c[2] = Lk[2] + b.z;
-          c[3] = Lk[3] + b.w;
-        }
-        // (M, c) o (M', c') = (M M', M c' + c)
-        auto compose = [&](const float* M2, const float* c2) {
-          float R[16], r[4];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q)
-              R[4 * i + q] = M[4 * i] * M2[q] + M[4 * i + 1] * M2[4 + q] + M[4 * i + 2] * M2[8 + q] +
-                             M[4 * i + 3] * M2[12 + q];
-            r[i] = M[4 * i] * c2[0] + M[4 * i + 1] * c2[1] + M[4 * i + 2] * c2[2] +
-                   M[4 * i + 3] * c2[3] + c[i];
-          }
-#pragma unroll
-          for (int i = 0; i < 16; ++i) M[i] = R[i];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) c[i] = r[i];
-        };
-        if (wid < 4) {
-          const int lane = tid & 31;
-#pragma unroll
-          for (int o = 1; o < 32; o <<= 1) {
-            float M2[16], c2[4];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) M2[i] = __shfl_up_sync(0xffffffffu, M[i], o);
-#pragma unroll
-            for (int i = 0; i < 4; ++i) c2[i] = __shfl_up_sync(0xffffffffu, c[i], o);
-            if (lane >= o) compose(M2, c2);
-          }
-          if (lane == 31) {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) rs.afm[20 * wid + i] = M[i];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) rs.afm[20 * wid + 16 + i] = c[i];
-          }
-        }
-        __syncthreads();
-        if (on) {
-          // the earlier warps' compositions, the latest one first (inside)
-          for (int v = wid - 1; v >= 0; --v) {
-            float M2[16], c2[4];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) M2[i] = rs.afm[20 * v + i];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) c2[i] = rs.afm[20 * v + 16 + i];
-            compose(M2, c2);
-          }
-        }
-        if (on) {
-          const float* L = rs.gs + (T - 1) * 10 + 3;  // Lq_{T-1}
-          const float l0 = L[0], l1 = L[1], l2 = L[2], l3 = L[3];
-          float* Lk = rs.gs + kk * 10 + 3;
-          float lo[4];
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-            lo[i] = M[4 * i] * l0 + M[4 * i + 1] * l1 + M[4 * i + 2] * l2 + M[4 * i + 3] * l3 + c[i];
-#pragma unroll
-          for (int i = 0; i < 4; ++i) Lk[i] = lo[i];
-        }
-      }
-      __syncthreads();
-      // (d) dS/du_k = the control part of J_k^T L_{k+1}
-      if (tid < T) {
-        float lam[10];
-#pragma unroll
-        for (int i = 0; i < 10; ++i) lam[i] = rs.gs[tid * 10 + i];
-        float gu[4] = {0.f, 0.f, 0.f, 0.f};
-        const float* stk = rs.st + (size_t)tid * 34;
-        rk4_vjp_stages(rs.xs + tid * 10, stk, stk + 10, stk + 20, stk + 30, u[tid], dp, lam, gu);
-        rs.g[tid] = make_float4(gu[0], gu[1], gu[2], gu[3]);
-      }
+    // backward: the suffix sums run up the threads, thread t taking step k = T - 1 - t
+    const int k = T - 1 - tid;
+    const bool on = k >= 0;
+    const float h = dp.dt;
+    const float3 zero = make_float3(0.f, 0.f, 0.f);
+    const float* g = rs.gs + (on ? k : 0) * 9;
+    const float3 gp = on ? make_float3(g[0], g[1], g[2]) : zero;
+    const float3 gv = on ? make_float3(g[3], g[4], g[5]) : zero;
+    const float3 tg = on ? make_float3(g[6], g[7], g[8]) : zero;
+    const float* q = rs.xs + (on ? k : 0) * 10 + 3;
+    const float3 lp = block_sum_scan3<kThreads / 32>(gp, rs.tot);              // Lp_{k+1}
+    const float3 lp2 = make_float3(lp.x - gp.x, lp.y - gp.y, lp.z - gp.z);     // Lp_{k+2}
+    const float3 lv = block_sum_scan3<kThreads / 32>(
+        make_float3(gv.x + h * lp2.x, gv.y + h * lp2.y, gv.z + h * lp2.z), rs.tot);
+    StepAdjoint sa;
+    float3 bt = zero;
+    if (on) bt = step_adjoint_translation(q, u[k], dp, lp, lv, sa);
+    const float3 ts = block_sum_scan3<kThreads / 32>(add3(tg, bt), rs.tot);
+    float4 un = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (on) {
+      const float4 uk = u[k];
+      const float3 tau = make_float3(ts.x - bt.x, ts.y - bt.y, ts.z - bt.z);   // tau_{k+1}
+      const float4 d = control_terms_grad(step_adjoint_controls(q, uk, dp, sa, tau), u, k, T, cp);
+      un = make_float4(fminf(fmaxf(uk.x - alpha * d.x, umin[0]), umax[0]),
+                       fminf(fmaxf(uk.y - alpha * d.y, umin[1]), umax[1]),
+                       fminf(fmaxf(uk.z - alpha * d.z, umin[2]), umax[2]),
+                       fminf(fmaxf(uk.w - alpha * d.w, umin[3]), umax[3]));
     }
-    __syncthreads();
-    // control terms, then the clamped step
-    if (tid < T) {
-      const int t = tid;
-      float4 a = rs.g[t];
-      const float4 ut = u[t];
-      if (t <= T - 2) {
-        a.x += 2.0f * cp.Q_c * ut.x; a.y += 2.0f * cp.Q_c * ut.y;
-        a.z += 2.0f * cp.Q_c * ut.z; a.w += 2.0f * cp.Q_c * ut.w;
-      }
-      if (t >= 1 && t <= T - 2) {
-        const float4 b = u[t - 1];
-        a.x += 2.0f * cp.Q_cd * (ut.x - b.x); a.y += 2.0f * cp.Q_cd * (ut.y - b.y);
-        a.z += 2.0f * cp.Q_cd * (ut.z - b.z); a.w += 2.0f * cp.Q_cd * (ut.w - b.w);
-      }
-      if (t + 1 >= 1 && t + 1 <= T - 2) {
-        const float4 c = u[t + 1];
-        a.x -= 2.0f * cp.Q_cd * (c.x - ut.x); a.y -= 2.0f * cp.Q_cd * (c.y - ut.y);
-        a.z -= 2.0f * cp.Q_cd * (c.z - ut.z); a.w -= 2.0f * cp.Q_cd * (c.w - ut.w);
-      }
-      rs.g[t] = a;
-    }
-    __syncthreads();
-    if (tid < T) {
-      const float4 a = u[tid], d = rs.g[tid];
-      u[tid] = make_float4(fminf(fmaxf(a.x - alpha * d.x, umin[0]), umax[0]),
-                           fminf(fmaxf(a.y - alpha * d.y, umin[1]), umax[1]),
-                           fminf(fmaxf(a.z - alpha * d.z, umin[2]), umax[2]),
-                           fminf(fmaxf(a.w - alpha * d.w, umin[3]), umax[3]));
-    }
+    __syncthreads();  // every step's neighbours read
+    if (on) u[k] = un;
     __syncthreads();
   }
 }

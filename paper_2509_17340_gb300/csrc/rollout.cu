@@ -1043,36 +1043,33 @@ static_assert(fused_update_fits(),
               "the split pass's shared memory holds the fused update and its refinement scratch");
 
 // One warp per control sequence: S(1) of its noise-free rollout and dS/dU.
-constexpr int kCgWarps = 4;
+// Small CTAs, so that a few thousand sequences spread evenly over the SMs.
+constexpr int kCgWarps = 2;
 
+template <bool kGrad>
 __global__ void __launch_bounds__(32 * kCgWarps) k_cost_grad(CostGradArgs a) {
-  __shared__ float4 s_u[kCgWarps][kMaxT];
-  __shared__ float4 s_g[kCgWarps][kMaxT];
-  __shared__ AdjScratch s_sc[kCgWarps];
+  extern __shared__ __align__(16) float cg_smem[];  // kCgWarps x cost_grad_words(T)
   const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = blockIdx.x * kCgWarps + wid;
   if (i >= a.n) return;  // uniform over the warp
   const int T = a.ctx.T;
-  for (int t = lane; t < T; t += 32) s_u[wid][t] = a.U[(size_t)i * T + t];
-  __syncwarp();
-  const float* guide = a.ctx.guides + (size_t)a.instance * T * 3;
-  float S;
-  if (a.G)
-    S = warp_cost_grad<true>(s_u[wid], s_g[wid], guide, T, a.ctx.x0, a.ctx.dyn, a.ctx.cost,
-                             a.ctx.grid, s_sc[wid], lane);
-  else
-    S = warp_cost_grad<false>(s_u[wid], s_g[wid], guide, T, a.ctx.x0, a.ctx.dyn, a.ctx.cost,
-                              a.ctx.grid, s_sc[wid], lane);
+  const float S = warp_cost_grad<kGrad>(a.U + (size_t)i * T, kGrad ? a.G + (size_t)i * T : nullptr,
+                                        a.ctx.guides + (size_t)a.instance * T * 3, T, a.ctx.x0, a.ctx.dyn,
+                                        a.ctx.cost, a.ctx.grid, cg_smem + wid * cost_grad_words(T), lane);
   if (lane == 0) a.S[i] = S;
-  if (a.G)
-    for (int t = lane; t < T; t += 32) a.G[(size_t)i * T + t] = s_g[wid][t];
 }
 
 }  // namespace
 
 cudaError_t launch_cost_grad(const CostGradArgs& a, cudaStream_t s) {
   if (a.n == 0) return cudaSuccess;
-  k_cost_grad<<<(a.n + kCgWarps - 1) / kCgWarps, 32 * kCgWarps, 0, s>>>(a);
+  // at most 18 KB at kMaxT, within the default limit
+  const size_t smem = sizeof(float) * kCgWarps * cost_grad_words(a.ctx.T);
+  const unsigned blocks = (unsigned)((a.n + kCgWarps - 1) / kCgWarps);
+  if (a.G)
+    k_cost_grad<true><<<blocks, 32 * kCgWarps, smem, s>>>(a);
+  else
+    k_cost_grad<false><<<blocks, 32 * kCgWarps, smem, s>>>(a);
   return cudaGetLastError();
 }
 

@@ -119,6 +119,40 @@ def test_cost_grad_matches_oracle_adjoint(aero, orc, name):
     pl.close()
 
 
+@pytest.mark.parametrize("T", [1, 2, 31, 32, 33, 64, 65, 128])
+def test_cost_grad_at_the_rounds_of_32_steps(aero, orc, T):
+    """One warp takes 32 steps at a time and carries the sums between the
+    rounds: horizons around their edges, and an odd number of sequences (two
+    warps per CTA)."""
+    import torch
+    w = _case("column", K=64, T=T, refine_steps=0)
+    P = w.params
+    pl, _, _, _ = _step(aero, w)
+    guides = pl.debug("GUIDES").reshape(P["E"], T, 3).astype(np.float64) + w.p0
+    pts = _oracle_pts(orc, w)
+    rng = np.random.default_rng(T)
+    hover = np.tile(np.array([P["mass"] * P["g"], 0, 0, 0], np.float32), (7, T, 1))
+    seqs = np.clip(hover + rng.normal(0, [0.3, 0.1, 0.1, 0.1], hover.shape), P["u_min"],
+                   P["u_max"]).astype(np.float32)
+    U = torch.from_numpy(seqs).cuda()
+    S = torch.empty(len(seqs), device="cuda")
+    G = torch.empty_like(U)
+    checked = 0
+    for e in (0, P["E"] - 1):
+        pl.cost_grad(e, U, S, G)
+        torch.cuda.synchronize()
+        for i, u in enumerate(seqs.astype(np.float64)):
+            if not _clear(orc, w, u, guides[e], pts)[0]:
+                continue
+            S_o, G_o = orc.cost_grad(x0_of(w), u, guides[e], w.goal.astype(np.float64), pts, P)
+            assert abs(float(S[i]) - S_o) <= TOL_COST_REL * abs(S_o), (e, i)
+            err = np.abs(G[i].cpu().numpy().astype(np.float64) - G_o).max()
+            assert err <= TOL_GRAD * np.abs(G_o).max() + 1e-3, (e, i, err, np.abs(G_o).max())
+            checked += 1
+    assert checked >= 1
+    pl.close()
+
+
 def test_autograd_function_uses_the_adjoint(aero):
     import torch
     w = _case("refined", K=256, T=20, refine_steps=0)
