@@ -3,7 +3,8 @@
 // step of the paper: it serves the gradient refinement of the updated nominals
 // before Stage II and the cost-and-gradient entry point.
 //
-// Every recurrence over the steps is a scan, one step per lane (thread).
+// Every recurrence over the steps is a scan, one step per lane (thread).  In the
+// cost-and-gradient kernel:
 // Forward: rollout_by_scans' prefix products and sums.  Backward, with
 // L_{k+1} = dS/dx_{k+1} (the state terms at x_{k+1} plus what flows back from
 // later steps):
@@ -466,47 +467,160 @@ __device__ float warp_cost_grad(const float4* __restrict__ U, float4* __restrict
 }
 
 // ---------------------------------------------------------------------------
-// Gradient refinement by a whole CTA (the update kernels), one step per
-// thread: the forward states by scans over the steps (rollout_by_scans), the
-// nearest point of every state (candidate lists cut into items of kRefItem
-// entries; a 64-bit atomic minimum of (squared distance bits, item index) keeps
-// the lowest item among equidistant points, the collision set's order), the
-// state terms and their gradients, three suffix sums for the adjoints, the
-// control terms and the clamped step.  Latency bound (one CTA per instance, the
-// barriers of the scans in a chain): five steps added 30 us to a planning step
-// of E = 8, K = 1024, T = 40 with the attitude adjoint as a scan of 4x4 affine
-// maps and the stages' reverse sweep twice, 20 us with the sums.
+// The RK4 step's stages and their reverse sweep (the refinement).
+// ---------------------------------------------------------------------------
+// xd = f(x, u) of the quadrotor model (Eq. dynamics) at a stage state.
+__device__ __forceinline__ void dyn_f(const float* x, float4 u, const DynParams& dp, float* xd) {
+  const float qw = x[3], qx = x[4], qy = x[5], qz = x[6];
+  xd[0] = x[7]; xd[1] = x[8]; xd[2] = x[9];
+  xd[3] = 0.5f * (-qx * u.y - qy * u.z - qz * u.w);
+  xd[4] = 0.5f * (qw * u.y + qy * u.w - qz * u.z);
+  xd[5] = 0.5f * (qw * u.z - qx * u.w + qz * u.y);
+  xd[6] = 0.5f * (qw * u.w + qx * u.z - qy * u.y);
+  float rx, ry, rz;
+  r_e3(qw, qx, qy, qz, rx, ry, rz);
+  const float f = u.x * dp.inv_mass;
+  xd[7] = f * rx; xd[8] = f * ry; xd[9] = f * rz - dp.g;
+}
+
+// w^T df/dx added to gx, w^T df/du added to gu, at stage state x.
+__device__ __forceinline__ void dyn_vjp(const float* x, float4 u, const DynParams& dp,
+                                        const float* w, float* gx, float* gu) {
+  const float qw = x[3], qx = x[4], qy = x[5], qz = x[6];
+  const float ox = u.y, oy = u.z, oz = u.w;
+  gx[7] += w[0]; gx[8] += w[1]; gx[9] += w[2];
+  const float W0 = 0.5f * w[3], W1 = 0.5f * w[4], W2 = 0.5f * w[5], W3 = 0.5f * w[6];
+  gx[3] += W1 * ox + W2 * oy + W3 * oz;
+  gx[4] += -W0 * ox - W2 * oz + W3 * oy;
+  gx[5] += -W0 * oy + W1 * oz - W3 * ox;
+  gx[6] += -W0 * oz - W1 * oy + W2 * ox;
+  gu[1] += -W0 * qx + W1 * qw + W2 * qz - W3 * qy;
+  gu[2] += -W0 * qy - W1 * qz + W2 * qw + W3 * qx;
+  gu[3] += -W0 * qz + W1 * qy - W2 * qx + W3 * qw;
+  const float V0 = w[7], V1 = w[8], V2 = w[9];
+  float rx, ry, rz;
+  r_e3(qw, qx, qy, qz, rx, ry, rz);
+  gu[0] += (V0 * rx + V1 * ry + V2 * rz) * dp.inv_mass;
+  const float s = u.x * dp.inv_mass;
+  gx[3] += s * (2.0f * qy * V0 - 2.0f * qx * V1);
+  gx[4] += s * (2.0f * qz * V0 - 2.0f * qw * V1 - 4.0f * qx * V2);
+  gx[5] += s * (2.0f * qw * V0 + 2.0f * qz * V1 - 4.0f * qy * V2);
+  gx[6] += s * (2.0f * qx * V0 + 2.0f * qy * V1);
+}
+
+// The stage states of one RK4 step from x with control u (Eq. dynamics):
+// t2 = x + h/2 k1, t3 = x + h/2 k2, t4 = x + h k3, and the quaternion before
+// renormalisation y = q + h/6 (k1 + 2 k2 + 2 k3 + k4) (quaternion part).
+__device__ __forceinline__ void rk4_stages(const float* x, float4 u, const DynParams& dp, float* t2,
+                                           float* t3, float* t4, float* y) {
+  const float h = dp.dt;
+  float k1[10], k2[10], k3[10], k4[10];
+  dyn_f(x, u, dp, k1);
+#pragma unroll
+  for (int i = 0; i < 10; ++i) t2[i] = x[i] + 0.5f * h * k1[i];
+  dyn_f(t2, u, dp, k2);
+#pragma unroll
+  for (int i = 0; i < 10; ++i) t3[i] = x[i] + 0.5f * h * k2[i];
+  dyn_f(t3, u, dp, k3);
+#pragma unroll
+  for (int i = 0; i < 10; ++i) t4[i] = x[i] + h * k3[i];
+  dyn_f(t4, u, dp, k4);
+#pragma unroll
+  for (int i = 0; i < 4; ++i)
+    y[i] = x[3 + i] + h * (1.0f / 6.0f) * (k1[3 + i] + 2.0f * k2[3 + i] + 2.0f * k3[3 + i] + k4[3 + i]);
+}
+
+// Reverse of one RK4 step given its stage states: lam holds dS/dx_{j+1} on
+// entry and dS/dx_j on return; gu gets dS/du_j from the dynamics.  Through the
+// renormalisation q+ = y/|y| (projection (I - q+ q+^T)/|y|), then the four
+// stages in reverse.
+__device__ __forceinline__ void rk4_vjp_stages(const float* x, const float* t2, const float* t3,
+                                               const float* t4, const float* y, float4 u,
+                                               const DynParams& dp, float* lam, float* gu) {
+  const float h = dp.dt;
+  const float inv = rsqrtf(y[0] * y[0] + y[1] * y[1] + y[2] * y[2] + y[3] * y[3]);
+  const float dot = (y[0] * lam[3] + y[1] * lam[4] + y[2] * lam[5] + y[3] * lam[6]) * inv;
+  float ly[10];
+#pragma unroll
+  for (int i = 0; i < 10; ++i) ly[i] = lam[i];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) ly[3 + i] = (lam[3 + i] - y[i] * inv * dot) * inv;
+  float l1[10], l2[10], l3[10], l4[10], lt[10];
+#pragma unroll
+  for (int i = 0; i < 10; ++i) {
+    lam[i] = ly[i];
+    l1[i] = h * (1.0f / 6.0f) * ly[i];
+    l2[i] = h * (1.0f / 3.0f) * ly[i];
+    l3[i] = l2[i];
+    l4[i] = l1[i];
+  }
+#pragma unroll
+  for (int i = 0; i < 10; ++i) lt[i] = 0.0f;
+  dyn_vjp(t4, u, dp, l4, lt, gu);
+#pragma unroll
+  for (int i = 0; i < 10; ++i) { lam[i] += lt[i]; l3[i] += h * lt[i]; lt[i] = 0.0f; }
+  dyn_vjp(t3, u, dp, l3, lt, gu);
+#pragma unroll
+  for (int i = 0; i < 10; ++i) { lam[i] += lt[i]; l2[i] += 0.5f * h * lt[i]; lt[i] = 0.0f; }
+  dyn_vjp(t2, u, dp, l2, lt, gu);
+#pragma unroll
+  for (int i = 0; i < 10; ++i) { lam[i] += lt[i]; l1[i] += 0.5f * h * lt[i]; }
+  dyn_vjp(x, u, dp, l1, lam, gu);
+}
+
+// ---------------------------------------------------------------------------
+// Gradient refinement by a whole CTA (the update kernels): the forward
+// states by scans over the steps (rollout_by_scans); the backward pass split
+// by dependence (suffix sums for the position and velocity adjoints, the 4x4
+// attitude recurrence on one thread, the vector-Jacobian products of every
+// step in parallel); everything else over the CTA: the stage states of every
+// step, the nearest point of every
+// state (candidate lists cut into items of kRefItem entries; a 64-bit atomic
+// minimum of (squared distance bits, item index) keeps the lowest item among
+// equidistant points, the collision set's order), the state terms and their
+// gradients, the control terms and the clamped step.  It keeps the stages' reverse
+// sweep and the affine attitude recurrence, not warp_cost_grad's sums: five steps
+// of 0.05 on gradients of up to 1e6 magnify a change of rounding (the refined nominals
+// moved by up to 1e-5 of their norm, past their error against 64 bits on some
+// inputs) and the sums saved 10 us of 74.
 // ---------------------------------------------------------------------------
 constexpr int kRefItem = 8;
 
 struct RefineScratch {
   float4* tot;               // warps: scan totals of the forward rollout
+  float4* g;                 // T: dS/du
   unsigned long long* key;   // T: (bits(d2) << 32) | item of the nearest point of x_{j+1}
   float4* near;              // T: that point (entries holding points: found by a second pass)
   int2* qrange;              // T: candidate range of each listed query
   int2* scan;                // warps: block-scan totals
   float* xs;                 // (T + 1) x 10: states x_0 .. x_T
-  float* gs;                 // T x 9: state-term gradients at x_{j+1} (gp, gv, part of tau)
+  float* st;                 // T x 34: stage states t2, t3, t4 and y of step j
+  float* gs;                 // T x 10: state-term gradients at x_{j+1}
   int* qitem;                // T + 1: first item of each listed query
   int* qslot;                // T: step of each listed query
+  float* afm;                // 4 x 20: the attitude adjoint scan's warp compositions
 };
 
 __host__ __device__ constexpr size_t refine_smem_bytes(int T, int warps) {
-  return 16 * (size_t)warps + 8 * (size_t)T + 16 * (size_t)T + 8 * (size_t)T + 8 * (size_t)warps +
-         4 * (size_t)(T + 1) * 10 + 4 * (size_t)T * 9 + 4 * (size_t)(T + 1) + 4 * (size_t)T;
+  return 16 * (size_t)warps + 16 * (size_t)T + 8 * (size_t)T + 16 * (size_t)T + 8 * (size_t)T + 8 * (size_t)warps +
+         4 * (size_t)(T + 1) * 10 + 4 * (size_t)T * 34 + 4 * (size_t)T * 10 + 4 * (size_t)(T + 1) +
+         4 * (size_t)T + 4 * 80;
 }
 
 __device__ __forceinline__ RefineScratch refine_layout(unsigned char* base, int T, int warps) {
   RefineScratch r;
   r.tot = reinterpret_cast<float4*>(base);
-  r.near = r.tot + warps;
-  r.key = reinterpret_cast<unsigned long long*>(r.near + T);
-  r.qrange = reinterpret_cast<int2*>(r.key + T);
+  r.g = r.tot + warps;
+  r.key = reinterpret_cast<unsigned long long*>(r.g + T);
+  r.near = reinterpret_cast<float4*>(r.key + T);
+  r.qrange = reinterpret_cast<int2*>(r.near + T);
   r.scan = r.qrange + T;
   r.xs = reinterpret_cast<float*>(r.scan + warps);
-  r.gs = r.xs + (size_t)(T + 1) * 10;
-  r.qitem = reinterpret_cast<int*>(r.gs + (size_t)T * 9);
+  r.st = r.xs + (size_t)(T + 1) * 10;
+  r.gs = r.st + (size_t)T * 34;
+  r.qitem = reinterpret_cast<int*>(r.gs + (size_t)T * 10);
   r.qslot = r.qitem + T + 1;
+  r.afm = reinterpret_cast<float*>(r.qslot + T);
   return r;
 }
 
@@ -525,9 +639,11 @@ __device__ void block_refine(float4* u, const float* guide, int T, const float* 
   for (int r = 0; r < steps; ++r) {
     // forward: the states x_0 .. x_T, by scans over the steps
     rollout_by_scans<kThreads / 32>(u, T, x0, dp, rs.xs, rs.tot);
-    // the candidate range of x_{tid+1}
+    // step tid: its stage states and the candidate range of x_{tid+1}
     int2 rg = make_int2(0, 0);
     if (tid < T) {
+      float* stj = rs.st + (size_t)tid * 34;
+      rk4_stages(rs.xs + tid * 10, u[tid], dp, stj, stj + 10, stj + 20, stj + 30);
       rs.key[tid] = none;
       const float* x1 = rs.xs + (tid + 1) * 10;
       rg = cell_range(x1[0], x1[1], x1[2], grid);
@@ -596,47 +712,194 @@ __device__ void block_refine(float4* u, const float* guide, int T, const float* 
       const float4 nearest = bi == 0xffffffffu ? make_float4(0.f, 0.f, 0.f, 0.f)
                              : grid.cand       ? __ldg(grid.pts + bi)
                                                : rs.near[tid];
-      const State x1 = state_load(rs.xs + (tid + 1) * 10);
-      float gs[10];
-      state_terms<true>(x1, guide[3 * tid], guide[3 * tid + 1], guide[3 * tid + 2], d2, nearest, cp,
-                        dmax2, gs);
-      const float3 t = vec_mul_conj(gs + 3, x1.q);
-      float* g = rs.gs + tid * 9;
-      g[0] = gs[0]; g[1] = gs[1]; g[2] = gs[2];
-      g[3] = gs[7]; g[4] = gs[8]; g[5] = gs[9];
-      g[6] = t.x; g[7] = t.y; g[8] = t.z;
+      state_terms<true>(state_load(rs.xs + (tid + 1) * 10), guide[3 * tid], guide[3 * tid + 1],
+                        guide[3 * tid + 2], d2, nearest, cp, dmax2, rs.gs + tid * 10);
     }
     __syncthreads();
-    // backward: the suffix sums run up the threads, thread t taking step k = T - 1 - t
-    const int k = T - 1 - tid;
-    const bool on = k >= 0;
-    const float h = dp.dt;
-    const float3 zero = make_float3(0.f, 0.f, 0.f);
-    const float* g = rs.gs + (on ? k : 0) * 9;
-    const float3 gp = on ? make_float3(g[0], g[1], g[2]) : zero;
-    const float3 gv = on ? make_float3(g[3], g[4], g[5]) : zero;
-    const float3 tg = on ? make_float3(g[6], g[7], g[8]) : zero;
-    const float* q = rs.xs + (on ? k : 0) * 10 + 3;
-    const float3 lp = block_sum_scan3<kThreads / 32>(gp, rs.tot);              // Lp_{k+1}
-    const float3 lp2 = make_float3(lp.x - gp.x, lp.y - gp.y, lp.z - gp.z);     // Lp_{k+2}
-    const float3 lv = block_sum_scan3<kThreads / 32>(
-        make_float3(gv.x + h * lp2.x, gv.y + h * lp2.y, gv.z + h * lp2.z), rs.tot);
-    StepAdjoint sa;
-    float3 bt = zero;
-    if (on) bt = step_adjoint_translation(q, u[k], dp, lp, lv, sa);
-    const float3 ts = block_sum_scan3<kThreads / 32>(add3(tg, bt), rs.tot);
-    float4 un = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (on) {
-      const float4 uk = u[k];
-      const float3 tau = make_float3(ts.x - bt.x, ts.y - bt.y, ts.z - bt.z);   // tau_{k+1}
-      const float4 d = control_terms_grad(step_adjoint_controls(q, uk, dp, sa, tau), u, k, T, cp);
-      un = make_float4(fminf(fmaxf(uk.x - alpha * d.x, umin[0]), umax[0]),
-                       fminf(fmaxf(uk.y - alpha * d.y, umin[1]), umax[1]),
-                       fminf(fmaxf(uk.z - alpha * d.z, umin[2]), umax[2]),
-                       fminf(fmaxf(uk.w - alpha * d.w, umin[3]), umax[3]));
+    // backward.  With L_{k+1} = dS/dx_{k+1} (the state terms at x_{k+1} plus
+    // what flows back from later steps), L_{k+1} = gs[k] + J_{k+1}^T L_{k+2},
+    // J the step Jacobian.  Positions feed only positions and velocities only
+    // positions and velocities, so the position and velocity parts are
+    // suffix sums: Lp_{k+1} = sum_{i >= k} gs_p[i], Lv_{k+1} = sum_{i >= k}
+    // (gs_v[i] + h Lp_{i+2}).  The attitude part is the linear recurrence
+    // Lq_{k+1} = gs_q[k] + b_{k+1} + A_{k+1}^T Lq_{k+2}: b the attitude part of
+    // J^T (Lp, 0, Lv) (the step's vector-Jacobian product, in parallel), A the
+    // 4x4 attitude Jacobian, whose transpose is applied in closed form: the
+    // unnormalised y = q (x) m, so A^T l = ((l - yh (yh . l)) / |y|) (x) conj(m),
+    // yh = y / |y|; one thread chains it.  Then every step's dS/du_k is the
+    // control part of J_k^T L_{k+1}, in parallel.
+    {
+      const float h = dp.dt;
+      // (a) the suffix sums, thread t taking step k = T - 1 - t
+      const int k = T - 1 - tid;
+      const bool on = tid < T;
+      const float* g = rs.gs + (on ? k : 0) * 10;
+      const float3 gp = on ? make_float3(g[0], g[1], g[2]) : make_float3(0.f, 0.f, 0.f);
+      const float3 gv = on ? make_float3(g[7], g[8], g[9]) : make_float3(0.f, 0.f, 0.f);
+      const float3 lp = block_sum_scan3<kThreads / 32>(gp, rs.tot);
+      const float3 lp2 = make_float3(lp.x - gp.x, lp.y - gp.y, lp.z - gp.z);  // Lp_{k+2}
+      const float3 lv = block_sum_scan3<kThreads / 32>(
+          make_float3(gv.x + h * lp2.x, gv.y + h * lp2.y, gv.z + h * lp2.z), rs.tot);
+      if (on) {
+        float* L = rs.gs + k * 10;
+        L[0] = lp.x; L[1] = lp.y; L[2] = lp.z;
+        L[7] = lv.x; L[8] = lv.y; L[9] = lv.z;
+      }
+      __syncthreads();
+      // (b) b_k for every step k = tid, into rs.g
+      if (tid < T) {
+        const float* L = rs.gs + tid * 10;
+        float lam[10] = {L[0], L[1], L[2], 0.f, 0.f, 0.f, 0.f, L[7], L[8], L[9]};
+        float gu[4] = {0.f, 0.f, 0.f, 0.f};
+        const float* stk = rs.st + (size_t)tid * 34;
+        rk4_vjp_stages(rs.xs + tid * 10, stk, stk + 10, stk + 20, stk + 30, u[tid], dp, lam, gu);
+        rs.g[tid] = make_float4(lam[3], lam[4], lam[5], lam[6]);
+      }
+      __syncthreads();
+      // (c) the attitude recurrence Lq_k = C_k + A_{k+1}^T Lq_{k+1} (k = T-2
+      // .. 0; C_k = gs_q[k] + b_{k+1}; Lq_{T-1} = gs_q[T-1]) is affine in Lq:
+      // thread t = T-2-k holds the map x -> C_k + M x (M = A_{k+1}^T as a 4x4
+      // matrix, its columns the images of the unit vectors), and an inclusive
+      // scan composes the maps, later ones outside, so that thread t ends with
+      // the composition that takes Lq_{T-1} to Lq_k.  T - 1 <= 127 maps: up to
+      // four warps, each carrying the earlier warps' compositions.
+      static_assert(kMaxT - 1 <= 128 && kThreads >= 128, "the attitude adjoint scan spans four warps");
+      {
+        const int kk = T - 2 - tid, wid = tid >> 5;
+        const bool on = kk >= 0;
+        float M[16], c[4];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) M[i] = (i % 5 == 0) ? 1.0f : 0.0f;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) c[i] = 0.0f;
+        if (on) {
+          const int j = kk + 1;  // A_j: the attitude Jacobian of step j
+          const float* y = rs.st + (size_t)j * 34 + 30;
+          const float inv = rsqrtf(y[0] * y[0] + y[1] * y[1] + y[2] * y[2] + y[3] * y[3]);
+          const float4 m = rk4_attitude_coefs(u[j], dp);
+          const float4 mc = make_float4(m.x, -m.y, -m.z, -m.w);
+#pragma unroll
+          for (int col = 0; col < 4; ++col) {
+            // A_j^T e_col = ((e_col - yh (yh . e_col)) / |y|) (x) conj(m)
+            const float d = y[col] * inv * inv;
+            const float4 pl = make_float4(((col == 0 ? 1.f : 0.f) - y[0] * d) * inv,
+                                          ((col == 1 ? 1.f : 0.f) - y[1] * d) * inv,
+                                          ((col == 2 ? 1.f : 0.f) - y[2] * d) * inv,
+                                          ((col == 3 ? 1.f : 0.f) - y[3] * d) * inv);
+            const float4 at = quat_mul4(pl, mc);
+            M[col] = at.x;
+            M[4 + col] = at.y;
+            M[8 + col] = at.z;
+            M[12 + col] = at.w;
+          }
+          const float* Lk = rs.gs + kk * 10 + 3;
+          const float4 b = rs.g[j];
+          c[0] = Lk[0] + b.x;
+          c[1] = Lk[1] + b.y;
+          c[2] = Lk[2] + b.z;
+          c[3] = Lk[3] + b.w;
+        }
+        // (M, c) o (M', c') = (M M', M c' + c)
+        auto compose = [&](const float* M2, const float* c2) {
+          float R[16], r[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+              R[4 * i + q] = M[4 * i] * M2[q] + M[4 * i + 1] * M2[4 + q] + M[4 * i + 2] * M2[8 + q] +
+                             M[4 * i + 3] * M2[12 + q];
+            r[i] = M[4 * i] * c2[0] + M[4 * i + 1] * c2[1] + M[4 * i + 2] * c2[2] +
+                   M[4 * i + 3] * c2[3] + c[i];
+          }
+#pragma unroll
+          for (int i = 0; i < 16; ++i) M[i] = R[i];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) c[i] = r[i];
+        };
+        if (wid < 4) {
+          const int lane = tid & 31;
+#pragma unroll
+          for (int o = 1; o < 32; o <<= 1) {
+            float M2[16], c2[4];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) M2[i] = __shfl_up_sync(0xffffffffu, M[i], o);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) c2[i] = __shfl_up_sync(0xffffffffu, c[i], o);
+            if (lane >= o) compose(M2, c2);
+          }
+          if (lane == 31) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i) rs.afm[20 * wid + i] = M[i];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) rs.afm[20 * wid + 16 + i] = c[i];
+          }
+        }
+        __syncthreads();
+        if (on) {
+          // the earlier warps' compositions, the latest one first (inside)
+          for (int v = wid - 1; v >= 0; --v) {
+            float M2[16], c2[4];
+#pragma unroll
+            for (int i = 0; i < 16; ++i) M2[i] = rs.afm[20 * v + i];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) c2[i] = rs.afm[20 * v + 16 + i];
+            compose(M2, c2);
+          }
+        }
+        if (on) {
+          const float* L = rs.gs + (T - 1) * 10 + 3;  // Lq_{T-1}
+          const float l0 = L[0], l1 = L[1], l2 = L[2], l3 = L[3];
+          float* Lk = rs.gs + kk * 10 + 3;
+          float lo[4];
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            lo[i] = M[4 * i] * l0 + M[4 * i + 1] * l1 + M[4 * i + 2] * l2 + M[4 * i + 3] * l3 + c[i];
+#pragma unroll
+          for (int i = 0; i < 4; ++i) Lk[i] = lo[i];
+        }
+      }
+      __syncthreads();
+      // (d) dS/du_k = the control part of J_k^T L_{k+1}
+      if (tid < T) {
+        float lam[10];
+#pragma unroll
+        for (int i = 0; i < 10; ++i) lam[i] = rs.gs[tid * 10 + i];
+        float gu[4] = {0.f, 0.f, 0.f, 0.f};
+        const float* stk = rs.st + (size_t)tid * 34;
+        rk4_vjp_stages(rs.xs + tid * 10, stk, stk + 10, stk + 20, stk + 30, u[tid], dp, lam, gu);
+        rs.g[tid] = make_float4(gu[0], gu[1], gu[2], gu[3]);
+      }
     }
-    __syncthreads();  // every step's neighbours read
-    if (on) u[k] = un;
+    __syncthreads();
+    // control terms, then the clamped step
+    if (tid < T) {
+      const int t = tid;
+      float4 a = rs.g[t];
+      const float4 ut = u[t];
+      if (t <= T - 2) {
+        a.x += 2.0f * cp.Q_c * ut.x; a.y += 2.0f * cp.Q_c * ut.y;
+        a.z += 2.0f * cp.Q_c * ut.z; a.w += 2.0f * cp.Q_c * ut.w;
+      }
+      if (t >= 1 && t <= T - 2) {
+        const float4 b = u[t - 1];
+        a.x += 2.0f * cp.Q_cd * (ut.x - b.x); a.y += 2.0f * cp.Q_cd * (ut.y - b.y);
+        a.z += 2.0f * cp.Q_cd * (ut.z - b.z); a.w += 2.0f * cp.Q_cd * (ut.w - b.w);
+      }
+      if (t + 1 >= 1 && t + 1 <= T - 2) {
+        const float4 c = u[t + 1];
+        a.x -= 2.0f * cp.Q_cd * (c.x - ut.x); a.y -= 2.0f * cp.Q_cd * (c.y - ut.y);
+        a.z -= 2.0f * cp.Q_cd * (c.z - ut.z); a.w -= 2.0f * cp.Q_cd * (c.w - ut.w);
+      }
+      rs.g[t] = a;
+    }
+    __syncthreads();
+    if (tid < T) {
+      const float4 a = u[tid], d = rs.g[tid];
+      u[tid] = make_float4(fminf(fmaxf(a.x - alpha * d.x, umin[0]), umax[0]),
+                           fminf(fmaxf(a.y - alpha * d.y, umin[1]), umax[1]),
+                           fminf(fmaxf(a.z - alpha * d.z, umin[2]), umax[2]),
+                           fminf(fmaxf(a.w - alpha * d.w, umin[3]), umax[3]));
+    }
     __syncthreads();
   }
 }
