@@ -457,6 +457,10 @@ void make_step_args(aero_planner* pl, const aero_state_t* x0, const float* cloud
   pa.filter = n >= kPartFilterPointsPerCone * (int64_t)a.ncell;
   pa.el_lo = p.el_lo;
   pa.el_inv = (float)p.fine_el / (p.el_hi - p.el_lo);
+  pa.az_scale = (float)p.fine_az * 0.159154943f;
+  // 1e-5 rad, and what the multiplication into units of cones rounds off
+  pa.az_eps = 1e-5f * pa.az_scale + 1e-6f * (float)p.fine_az;
+  pa.el_eps = 1e-5f * pa.el_inv + 1e-6f * ((float)p.fine_el + std::fabs(p.el_lo) * pa.el_inv);
   pa.keys = pl->keys;
   pa.item_flag = a.raw ? pl->item_flag : nullptr;
   pa.counts = pl->part_counts;

@@ -60,7 +60,9 @@ struct PartitionArgs {
   int A, El;
   int check_lo, check_hi;
   int filter;      // read a cone's key before its atomic minimum (dense clouds)
-  float el_lo, el_inv;  // elevation span start and cones per radian (bin guesses only)
+  float el_lo, el_inv;  // elevation span start and cones per radian
+  float az_scale;       // azimuth cones per radian
+  float az_eps, el_eps; // distance to an edge, in cones, from which an angle guess decides the bin
   unsigned long long* keys;
   int* item_flag;  // collision set = every kept point: 1 where the point is kept, else 0
   int2* counts;    // per block (batched: per chunk of points): {non-finite points, kept points}
