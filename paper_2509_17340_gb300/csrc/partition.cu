@@ -384,11 +384,19 @@ __device__ __forceinline__ void cand_task(const CandArgs& a, int64_t it, int lan
   const int z1 = min(__float2int_rd((pz + g.reach - g.origin) * g.inv_h), g.G - 1);
   const int nx = x1 - x0 + 1, ny = y1 - y0 + 1, nz = z1 - z0 + 1;
   if (nx <= 0 || ny <= 0 || nz <= 0) return;
-  const int ncand = nx * ny * nz;
+  const int nxy = nx * ny, ncand = nxy * nz;
+  // o / nx and o / (nx ny) by multiplication, exact while o times the divisor stays
+  // below 2^16 (blocks of up to 9^3 cells; 5^3 and 6^3 with cells of d_max / 2).  The
+  // passes are bound by instruction issue: with runtime divisions per cell the
+  // batched count and scatter of 64 planners took 86 and 174 us instead of 78 and
+  // 157, those of 178,000 kept points 105 and 159 instead of 93 and 151.
+  const bool by_mul = ncand <= 65536 / nxy;
+  const int inv_x = (65535 + nx) / nx, inv_xy = (65535 + nxy) / nxy;
   // the cell of block offset o if the point is within reach of its box, else -1
   auto cell_of = [&](int o) {
     if (o >= ncand) return -1;
-    const int x = x0 + o % nx, y = y0 + (o / nx) % ny, z = z0 + o / (nx * ny);
+    const int qx = by_mul ? o * inv_x >> 16 : o / nx, qz = by_mul ? o * inv_xy >> 16 : o / nxy;
+    const int x = x0 + o - qx * nx, y = y0 + qx - qz * ny, z = z0 + qz;
     const float d2 = gap2(px, g.origin + x * g.h, g.h) + gap2(py, g.origin + y * g.h, g.h) +
                      gap2(pz, g.origin + z * g.h, g.h);
     if (d2 >= r2) return -1;
