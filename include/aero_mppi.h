@@ -70,7 +70,8 @@ extern "C" {
 #define AERO_DBG_GRID_META 6     /* int32 [4] = {G, n_entries, capacity, 0} then float [4] =
                                     {origin, h, reach, 0}: G^3 cells of edge h from origin
                                     (all axes); cell c lists every collision point closer
-                                    than reach (>= d_max) to its box */
+                                    than reach (>= d_max) to its box (where the step pruned
+                                    its lists, the whole lists, the entries left out first) */
 #define AERO_DBG_GRID_START 7    /* int32 [G*G*G + 1]: first entry of cell (z*G+y)*G+x */
 #define AERO_DBG_GRID_POINTS 8   /* float4 [n_entries]: candidate points - p0, grouped by cell */
 #define AERO_DBG_SAMPLE_COSTS 9  /* float [E][K]: S(1) of every sample, last iteration */
@@ -433,7 +434,7 @@ int aero_sync_status(aero_planner_t* planner, void* stream);
  * launches[AERO_STAGE_COUNT], and starts over.
  *   AERO_STAGE_PARTITION: workspace clears + fine partition (Sec. IV-A.1)
  *   AERO_STAGE_GRID: P_f / grid counts, coarse argmax + anchors + guides with the
- *                    grid scan, grid scatter (Sec. IV-A.2, IV-B)
+ *                    grid scan, grid scatter, list pruning (Sec. IV-A.2, IV-B)
  *   AERO_STAGE_ROLLOUT: sampling, rollouts and S(1) (Sec. III-B, IV-C)
  *   AERO_STAGE_UPDATE: weights, update, Stage II and selection */
 #define AERO_STAGE_PARTITION 0

@@ -590,7 +590,6 @@ struct RefineScratch {
   float4* tot;               // warps: scan totals of the forward rollout
   float4* g;                 // T: dS/du
   unsigned long long* key;   // T: (bits(d2) << 32) | item of the nearest point of x_{j+1}
-  float4* near;              // T: that point (entries holding points: found by a second pass)
   int2* qrange;              // T: candidate range of each listed query
   int2* scan;                // warps: block-scan totals
   float* xs;                 // (T + 1) x 10: states x_0 .. x_T
@@ -602,7 +601,7 @@ struct RefineScratch {
 };
 
 __host__ __device__ constexpr size_t refine_smem_bytes(int T, int warps) {
-  return 16 * (size_t)warps + 16 * (size_t)T + 8 * (size_t)T + 16 * (size_t)T + 8 * (size_t)T + 8 * (size_t)warps +
+  return 16 * (size_t)warps + 16 * (size_t)T + 8 * (size_t)T + 8 * (size_t)T + 8 * (size_t)warps +
          4 * (size_t)(T + 1) * 10 + 4 * (size_t)T * 34 + 4 * (size_t)T * 10 + 4 * (size_t)(T + 1) +
          4 * (size_t)T + 4 * 80;
 }
@@ -612,8 +611,7 @@ __device__ __forceinline__ RefineScratch refine_layout(unsigned char* base, int 
   r.tot = reinterpret_cast<float4*>(base);
   r.g = r.tot + warps;
   r.key = reinterpret_cast<unsigned long long*>(r.g + T);
-  r.near = reinterpret_cast<float4*>(r.key + T);
-  r.qrange = reinterpret_cast<int2*>(r.near + T);
+  r.qrange = reinterpret_cast<int2*>(r.key + T);
   r.scan = r.qrange + T;
   r.xs = reinterpret_cast<float*>(r.scan + warps);
   r.st = r.xs + (size_t)(T + 1) * 10;
@@ -657,18 +655,18 @@ __device__ void block_refine(float4* u, const float* guide, int T, const float* 
       rs.qslot[off.x] = tid;
     }
     __syncthreads();
-    // the nearest point of a listed query's item of entries: (squared
-    // distance, item index) of the point of lowest (distance, item), and the point
-    auto item_min = [&](int it, int& j, float& best, int& bitem, float4& bp) {
+    // every item of entries of a listed query: its (squared distance, item index)
+    // pair of lowest (distance, item) into the query's minimum
+    for (int it = tid; it < total.y; it += kThreads) {
       const int lo = item_owner(rs.qitem, total.x, it);
       const int2 q = rs.qrange[lo];
-      j = rs.qslot[lo];
+      const int j = rs.qslot[lo];
       const int first = (it - rs.qitem[lo]) * kRefItem;
       const int n = q.y - first < kRefItem ? q.y - first : kRefItem;
-      best = dmax2;
-      bitem = -1;
-      if (!AERO_CHECK(j < T && first >= 0 && n > 0 && q.x >= 0, kChkQuery)) return;
+      if (!AERO_CHECK(j < T && first >= 0 && n > 0 && q.x >= 0, kChkQuery)) continue;
       const float* x1 = rs.xs + (j + 1) * 10;
+      float best = dmax2;
+      int bitem = -1;
       for (int c = 0; c < n; ++c) {
         const float4 p = grid_point(grid, q.x + first + c);
         const float d2 = dist2_to(p, x1[0], x1[1], x1[2]);
@@ -676,42 +674,18 @@ __device__ void block_refine(float4* u, const float* guide, int T, const float* 
         if (d2 < best || (d2 == best && bitem >= 0 && item < bitem)) {
           best = d2;
           bitem = item;
-          bp = p;
         }
       }
-    };
-    for (int it = tid; it < total.y; it += kThreads) {
-      int j, bitem;
-      float best;
-      float4 bp;
-      item_min(it, j, best, bitem, bp);
       if (bitem >= 0)
         atomicMin(rs.key + j, ((unsigned long long)__float_as_uint(best) << 32) | (unsigned)bitem);
     }
     __syncthreads();
-    if (!grid.cand) {
-      // entries holding the points: the winner's point from the item that
-      // holds the winning (distance, item) pair
-      for (int it = tid; it < total.y; it += kThreads) {
-        int j, bitem;
-        float best;
-        float4 bp;
-        item_min(it, j, best, bitem, bp);
-        if (bitem >= 0 &&
-            rs.key[j] == (((unsigned long long)__float_as_uint(best) << 32) | (unsigned)bitem))
-          rs.near[j] = bp;
-      }
-      __syncthreads();
-    }
     // state-term gradients at x_{tid+1}
     if (tid < T) {
       const unsigned long long kk = rs.key[tid];
       const float d2 = __uint_as_float((unsigned)(kk >> 32));
       const unsigned bi = (unsigned)kk;
-      // entries holding item indices: the item's point directly
-      const float4 nearest = bi == 0xffffffffu ? make_float4(0.f, 0.f, 0.f, 0.f)
-                             : grid.cand       ? __ldg(grid.pts + bi)
-                                               : rs.near[tid];
+      const float4 nearest = bi == 0xffffffffu ? make_float4(0.f, 0.f, 0.f, 0.f) : __ldg(grid.pts + bi);
       state_terms<true>(state_load(rs.xs + (tid + 1) * 10), guide[3 * tid], guide[3 * tid + 1],
                         guide[3 * tid + 2], d2, nearest, cp, dmax2, rs.gs + tid * 10);
     }

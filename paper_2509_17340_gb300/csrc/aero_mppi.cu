@@ -133,9 +133,8 @@ struct aero_planner {
   int* grid_local = nullptr;  // G^3 + 1 tile-local exclusive prefix
   int* tile_sum = nullptr;
   int* tile_off = nullptr;
-  float4* cand = nullptr;     // candidate entries: points, or item indices (as uint32)
-  float4* cand_pts = nullptr; // collision point of every item, minus p0 (index entries)
-  bool last_idx_entries = false;  // the last step's entries were item indices
+  uint32_t* cand = nullptr;   // candidate entries: item indices
+  float4* cand_pts = nullptr; // collision point of every item, minus p0
   int2* grid_range = nullptr; // G^3 {first entry, count}
   int cand_cap = 0;
   int grid_max = kGridMax;    // cells per axis the grid arrays can hold
@@ -201,8 +200,13 @@ constexpr int kFineDup = 216, kCoarseDup = 27;
 // atomic minimum: in dense clouds most points cannot lower their cone's key
 constexpr int64_t kPartFilterPointsPerCone = 32;
 // lists longer than this are scanned by the whole warp in the one-lane pass
-// when every kept point is the collision set
+// when every kept point is the collision set and its lists are not pruned
 constexpr int kWarpListThreshold = 8;
+// when lists are pruned (prunes_lists)
+constexpr int64_t kPruneStepsPerPoint = 14, kPruneSteps = 12000000;
+constexpr int64_t kPruneDenseSteps = 100000, kPruneDensePointsPerCone = 16;
+constexpr int kPruneDenseEntries = 131072, kPruneDenseEntriesPerCell = 2;
+constexpr int64_t kPruneBatchSteps = 400000;
 
 int cuda_fail(cudaError_t e) {
   if (e == cudaSuccess) return AERO_OK;
@@ -417,8 +421,8 @@ int lanes_of(const aero_params_t& p, int64_t quad_max) {
 
 void make_step_args(aero_planner* pl, const aero_state_t* x0, const float* cloud, int64_t n,
                     const float* goal, const aero_params_t& p, float* u_nom, float* u_best,
-                    float* cand, int32_t* best_idx, int lanes, bool coarse, bool idx_entries,
-                    StepArgs& a, int samples_per_cta = kRolloutThreads) {
+                    float* cand, int32_t* best_idx, int lanes, bool coarse, StepArgs& a,
+                    int samples_per_cta = kRolloutThreads) {
   a.ncell = p.fine_az * p.fine_el;
   // the edge tables depend only on the partition geometry: recomputed when it changes
   if (!pl->tab_valid || pl->tab_A != p.fine_az || pl->tab_El != p.fine_el || pl->tab_lo != p.el_lo ||
@@ -477,9 +481,8 @@ void make_step_args(aero_planner* pl, const aero_state_t* x0, const float* cloud
   ca.fill = pl->grid_fill;
   ca.local = pl->grid_local;
   ca.tile_off = pl->tile_off;
-  ca.cand = idx_entries ? reinterpret_cast<uint32_t*>(pl->cand) : nullptr;
-  ca.pts = idx_entries ? pl->cand_pts : nullptr;
-  ca.cand4 = idx_entries ? nullptr : pl->cand;
+  ca.cand = pl->cand;
+  ca.pts = pl->cand_pts;
   ca.status = pl->status;
   ca.reset_keys = nullptr;
 
@@ -525,8 +528,7 @@ void make_step_args(aero_planner* pl, const aero_state_t* x0, const float* cloud
   for (int i = 0; i < 3; ++i) cp.v_goal[i] = p.v_goal[i];
   for (int i = 0; i < 4; ++i) cp.q_goal[i] = p.q_goal[i];
   DynParams dp{p.dt, 1.0f / p.mass, p.g};
-  GridView gv{pl->grid_range, ca.cand, idx_entries ? pl->cand_pts : pl->cand, a.grid.G, a.grid.origin,
-              a.grid.inv_h};
+  GridView gv{pl->grid_range, pl->cand, pl->cand_pts, a.grid.G, a.grid.origin, a.grid.inv_h};
   const float x0v[10] = {0.0f, 0.0f, 0.0f, x0->q[0], x0->q[1], x0->q[2], x0->q[3],
                          x0->v[0], x0->v[1], x0->v[2]};
   a.lanes = lanes;
@@ -540,9 +542,6 @@ void make_step_args(aero_planner* pl, const aero_state_t* x0, const float* cloud
   ra.T = p.T;
   ra.nb = a.nb;
   ra.lanes_per_sample = lanes;
-  // every kept point as the collision set: lists of tens to hundreds of
-  // entries, uneven across a warp's queries; P_f's are short (a few entries)
-  ra.list_thr = a.raw ? kWarpListThreshold : 0;
   ra.inv_lambda = 1.0f / p.lambda;
   for (int c = 0; c < 4; ++c) {
     ra.sigma[c] = p.sigma[c];
@@ -600,6 +599,22 @@ void make_step_args(aero_planner* pl, const aero_state_t* x0, const float* cloud
   ra.done = ua.done;
 }
 
+// Whether a single planner's step prunes its candidate lists (k_grid_prune), and from
+// how many entries in all.  Pruning takes time by the entries, what it saves goes by
+// the sample-steps.  Every kept point: 178,000 points cost 320 us and save 0.12 ns and
+// more per sample-step, so from 14 sample-steps per point on.  P_f of a sparse
+// scene (555,000 entries, 36 us): 0.004 ns, so from 12 M sample-steps on.  P_f of a
+// dense one (0.2 to 0.8 ns) from 100,000 on; that it is dense is likely where the
+// cloud has 16 points per cone, and decided on the device by two entries per cell.
+bool prunes_lists(const aero_params_t& p, int64_t n, const StepArgs& a, int& min_total) {
+  const int64_t steps = (int64_t)p.E * p.K * p.T * p.iters;
+  min_total = 0;
+  if (a.raw) return steps >= kPruneStepsPerPoint * n;
+  if (steps >= kPruneSteps) return true;
+  min_total = std::max(kPruneDenseEntries, kPruneDenseEntriesPerCell * a.gcells);
+  return steps >= kPruneDenseSteps && n >= kPruneDensePointsPerCone * a.ncell;
+}
+
 // The planner's state after a step has been enqueued.
 void note_step(aero_planner* pl, const aero_params_t& p, const StepArgs& a) {
   pl->last_ctx = a.ua;
@@ -607,7 +622,6 @@ void note_step(aero_planner* pl, const aero_params_t& p, const StepArgs& a) {
   pl->have_step = true;
   pl->last = p;
   pl->last_grid = a.grid;
-  pl->last_idx_entries = a.ca.cand != nullptr;
   pl->last_ntiles = a.ntiles;
   pl->last_nb = a.nb;
   pl->last_part_slots = partition_blocks(a.pa.n);
@@ -642,7 +656,7 @@ int enqueue_step(aero_planner* pl, const aero_state_t* x0, const float* cloud, i
                  float* cand, int32_t* best_idx, cudaStream_t s, const float* mapped = nullptr) {
   StepArgs a;
   make_step_args(pl, x0, cloud, n, goal, p, u_nom, u_best, cand, best_idx,
-                 lanes_of(p, kQuadMaxSamples), false, true, a);
+                 lanes_of(p, kQuadMaxSamples), false, a);
   if (mapped) {
     a.pa.cloud = mapped;
     a.pa.copy_to = const_cast<float*>(cloud);
@@ -696,7 +710,7 @@ int enqueue_step(aero_planner* pl, const aero_state_t* x0, const float* cloud, i
     prof->launches[AERO_STAGE_ROLLOUT] = p.iters;
     prof->launches[AERO_STAGE_UPDATE] = rollout_runs_update(a.ra) ? 0 : p.iters;
   }
-  // count pass + coarse argmax, scan + goal cone/anchors/guides, scatter + cell ranges
+  // count pass + coarse argmax, scan + goal cone/anchors/guides, scatter + cell ranges, pruning
   if ((e = launch_grid_count(a.ca, a.ga, s)) != cudaSuccess) return cuda_fail(e);
   if ((e = launch_grid_scan(pl->grid_count, pl->grid_fill, pl->grid_local, pl->tile_sum,
                             pl->tile_off, a.gcells + 1, a.ntiles, nullptr, a.ga, pl->d_tab, s)) !=
@@ -705,6 +719,17 @@ int enqueue_step(aero_planner* pl, const aero_state_t* x0, const float* cloud, i
   if ((e = launch_grid_scatter(a.ca, pl->grid_range, a.gcells, pl->tile_sum, pl->tile_off,
                                a.ntiles, s)) != cudaSuccess)
     return cuda_fail(e);
+  int min_total = 0;
+  const bool prune = prunes_lists(p, n, a, min_total);
+  // every kept point as the collision set, unpruned: lists of tens to hundreds of
+  // entries, uneven across a warp's queries
+  a.ra.list_thr = a.raw && !prune ? kWarpListThreshold : 0;
+  if (prune) {
+    const PruneArgs pr{pl->cand, pl->cand_pts, pl->grid_range, (int)a.n_items, a.gcells, 0,
+                       min_total > 0 ? pl->tile_off + a.ntiles : nullptr, min_total, a.grid};
+    if ((e = launch_grid_prune(pr, s)) != cudaSuccess) return cuda_fail(e);
+    if (prof) ++prof->launches[AERO_STAGE_GRID];
+  }
   mark(AERO_STAGE_GRID, 3);
 
   const uint32_t ctr_base = a.ra.ctr3;
@@ -830,7 +855,7 @@ int create_planner(const aero_limits_t* limits, aero_planner_t** out, bool batch
   chk(alloc(&pl->grid_local, kGridCellsMax + 1));
   chk(alloc(&pl->tile_sum, kMaxTiles));
   chk(alloc(&pl->tile_off, kMaxTiles + 1));
-  chk(dev_malloc((void**)&pl->cand, (batch_slot ? sizeof(float4) : sizeof(uint32_t)) * (size_t)(cap > 0 ? cap : 1)));
+  chk(alloc(&pl->cand, cap));
   chk(alloc(&pl->cand_pts, std::max<int64_t>(L.fine_cells_max, pl->raw_max)));
   chk(alloc(&pl->grid_range, kGridCellsMax));
   chk(alloc(&pl->partials, (size_t)L.E_max * nbmax * (4 + 4 * L.T_max)));
@@ -1017,7 +1042,6 @@ int aero_get_debug(aero_planner_t* pl, int32_t what, void* dst, size_t bytes, vo
       const size_t ne = (size_t)(n_entries < g.cap ? n_entries : g.cap);
       const size_t need = sizeof(float4) * ne;
       if (bytes < need) return AERO_ERR_INVALID_ARG;
-      if (!pl->last_idx_entries) return cuda_fail(cudaMemcpy(dst, pl->cand, need, cudaMemcpyDefault));
       const size_t n_items = (size_t)std::max<int64_t>(pl->lim.fine_cells_max, pl->raw_max);
       std::vector<uint32_t> idx(ne);
       std::vector<float4> pts(n_items), out(ne);
@@ -1182,7 +1206,7 @@ constexpr size_t kNaBytes =
     align256(8 * (size_t)kNaCells) + align256(4 * (size_t)kNaCells) + align256(4 * (kNaE + 1)) +
     align256(4 * 3 * kNaE) + align256(4 * 3 * (size_t)kNaE * kNaT) + align256(4 * (size_t)kNaPoints) +
     3 * align256(4 * ((size_t)kNaGridCells + 1)) + align256(4 * (size_t)kNaTiles) +
-    align256(4 * ((size_t)kNaTiles + 1)) + align256(16 * (size_t)kNaCand) +
+    align256(4 * ((size_t)kNaTiles + 1)) + align256(4 * (size_t)kNaCand) +
     align256(16 * (size_t)std::max<int64_t>(kNaCells, kNaPoints)) +
     align256(8 * (size_t)kNaGridCells) +
     align256(4 * (size_t)kNaE * kNaNb * (4 + 4 * kNaT)) + align256(4 * (size_t)kNaE * kNaK) +
@@ -1253,7 +1277,7 @@ void noalloc_carve(unsigned char* base, aero_planner& pl) {
   pl.grid_local = reinterpret_cast<int*>(take(4 * ((size_t)kNaGridCells + 1)));
   pl.tile_sum = reinterpret_cast<int*>(take(4 * (size_t)kNaTiles));
   pl.tile_off = reinterpret_cast<int*>(take(4 * ((size_t)kNaTiles + 1)));
-  pl.cand = reinterpret_cast<float4*>(take(16 * (size_t)kNaCand));
+  pl.cand = reinterpret_cast<uint32_t*>(take(4 * (size_t)kNaCand));
   pl.cand_pts = reinterpret_cast<float4*>(take(16 * (size_t)std::max<int64_t>(kNaCells, kNaPoints)));
   pl.grid_range = reinterpret_cast<int2*>(take(8 * (size_t)kNaGridCells));
   pl.cand_cap = kNaCand;
@@ -1348,7 +1372,7 @@ struct aero_batch {
   aero_batch_config_t cfg{0, 0, 1, 0, 0};
   int last_n = 0;  // items of the last call (debug copies)
   // resident CTAs per SM of the batched kernels
-  int occ_grid[4] = {1, 1, 1, 1};  // partition, count, scan, scatter
+  int occ_grid[5] = {1, 1, 1, 1, 1};  // partition, count, scan, scatter, prune
   // rollout (1 lane), rollout (4 lanes), update, rollout (1 lane, 6/SM), rollout (1 lane, 64
   // samples per CTA), rollout (1 lane, 256 samples per CTA)
   int occ_roll[6] = {1, 1, 1, 1, 1, 1};
@@ -1372,7 +1396,7 @@ struct aero_batch {
   std::vector<TabKey> tab_key;
   // instantiated graphs, one per shape and configuration
   struct Graph {
-    int n, max_iters, has1, has4;
+    int n, max_iters, has1, has4, prune;
     aero_batch_config_t cfg;
     cudaGraphExec_t exec;
   };
@@ -1469,13 +1493,13 @@ bool same_cfg(const aero_batch_config_t& a, const aero_batch_config_t& b) {
          spc_of(a) == spc_of(b);
 }
 
-// The graph of one call shape: the four grid-stage launches, then per
+// The graph of one call shape: the five grid-stage launches, then per
 // iteration the Stage I launch(es) -- both lane widths side by side when both
 // occur -- and the update.
-cudaError_t batch_graph(aero_batch* b, int n, int max_iters, int has1, int has4,
+cudaError_t batch_graph(aero_batch* b, int n, int max_iters, int has1, int has4, int prune,
                         const aero_batch_config_t& cfg, cudaGraphExec_t* out) {
   for (auto& g : b->graphs)
-    if (g.n == n && g.max_iters == max_iters && g.has1 == has1 && g.has4 == has4 &&
+    if (g.n == n && g.max_iters == max_iters && g.has1 == has1 && g.has4 == has4 && g.prune == prune &&
         same_cfg(g.cfg, cfg)) {
       *out = g.exec;
       return cudaSuccess;
@@ -1502,6 +1526,7 @@ cudaError_t batch_graph(aero_batch* b, int n, int max_iters, int has1, int has4,
   if (le == cudaSuccess) le = launch_batch_count(v, S * b->occ_grid[1], c);
   if (le == cudaSuccess) le = launch_batch_scan(v, S * b->occ_grid[2], c);
   if (le == cudaSuccess) le = launch_batch_scatter(v, S * b->occ_grid[3], c);
+  if (le == cudaSuccess && prune) le = launch_batch_prune(v, S * b->occ_grid[4], c);
   for (int it = 0; it < max_iters && le == cudaSuccess; ++it) {
     if (has1 && has4) {
       le = cudaEventRecord(b->fork, c);
@@ -1529,7 +1554,7 @@ cudaError_t batch_graph(aero_batch* b, int n, int max_iters, int has1, int has4,
   e = cudaGraphInstantiate(&exec, graph, 0);
   cudaGraphDestroy(graph);
   if (e != cudaSuccess) return e;
-  b->graphs.push_back({n, max_iters, has1, has4, cfg, exec});
+  b->graphs.push_back({n, max_iters, has1, has4, prune, cfg, exec});
   *out = exec;
   return cudaSuccess;
 }
@@ -1558,6 +1583,7 @@ int batch_enqueue(aero_batch* b, const aero_batch_item_t* items, int n, cudaStre
   std::vector<int> lanes(n), T(n);
   std::vector<int> tab_changed;
   int max_iters = 0, has1 = 0, has4 = 0;
+  int64_t steps = 0;  // sample-steps of all items: lists are pruned from kPruneBatchSteps per item on
   for (int k = 0; k < kPreCount; ++k) pre[k * (n + 1)] = 0;
   for (int i = 0; i < n; ++i) {
     const aero_batch_item_t& it = items[i];
@@ -1576,7 +1602,7 @@ int batch_enqueue(aero_batch* b, const aero_batch_item_t* items, int n, cudaStre
     }
     StepArgs a;
     make_step_args(pl, &it.x0, it.cloud_xyz, it.n_points, it.goal, p, u_nom, u_best, cand, best,
-                   lanes_of(p, cfg.quad_max_samples), cfg.coarse_cells != 0, false, a, spc_of(cfg));
+                   lanes_of(p, cfg.quad_max_samples), cfg.coarse_cells != 0, a, spc_of(cfg));
     BatchItem& bi = hi[i];
     bi.pa = a.pa;
     bi.ca = a.ca;
@@ -1612,11 +1638,13 @@ int batch_enqueue(aero_batch* b, const aero_batch_item_t* items, int n, cudaStre
     set(kPreCoarse, (long long)a.ga.Ac * a.ga.Ec);
     set(kPreTiles, a.ntiles);
     set(kPreCells, (long long)a.gcells + bi.raw_keys);
+    set(kPrePrune, (a.gcells + kPruneCells - 1) / kPruneCells);
     set(kPreUpdate, p.E);
     roll_units[i] = (long long)p.E * a.nb;
     meta[i] = {a.grid, a.ntiles, a.nb};
     lanes[i] = a.lanes;
     T[i] = p.T;
+    steps += (int64_t)p.E * p.K * p.T * p.iters;
     if (p.iters > max_iters) max_iters = p.iters;
     (a.lanes == 4 ? has4 : has1) = 1;
   }
@@ -1639,7 +1667,7 @@ int batch_enqueue(aero_batch* b, const aero_batch_item_t* items, int n, cudaStre
   }
 
   cudaGraphExec_t exec = nullptr;
-  if ((e = batch_graph(b, n, max_iters, has1, has4, cfg, &exec)) != cudaSuccess) return cuda_fail(e);
+  if ((e = batch_graph(b, n, max_iters, has1, has4, steps >= kPruneBatchSteps * n, cfg, &exec)) != cudaSuccess) return cuda_fail(e);
   // workspaces whose counts or keys may be stale (new slot, interrupted step)
   for (int i = 0; i < n; ++i) {
     aero_planner* pl = b->planners[i];
@@ -1669,7 +1697,6 @@ int batch_enqueue(aero_batch* b, const aero_batch_item_t* items, int n, cudaStre
     pl->have_step = true;
     pl->last = items[i].params;
     pl->last_grid = meta[i].grid;
-    pl->last_idx_entries = false;
     pl->last_ntiles = meta[i].ntiles;
     pl->last_part_slots = (int)((items[i].n_points + kPartChunk - 1) / kPartChunk);
     pl->last_n_points = items[i].n_points;

@@ -401,24 +401,14 @@ __device__ __forceinline__ float dist2_to(const float4 q, float px, float py, fl
   return ax * ax + ay * ay + az * az;
 }
 
-// The collision point of candidate entry e of the grid (either form); its w
-// holds the bits of the point's item index (the position of the point in the
-// collision set: the fine cone of a P_f point, the index of a kept point).
+// The collision point of candidate entry e of the grid; its w holds the bits of
+// the point's item index (the position of the point in the collision set: the fine
+// cone of a P_f point, the index of a kept point).
 __device__ __forceinline__ float4 grid_point(const GridView& g, int e) {
-  return g.cand ? __ldg(g.pts + __ldg(g.cand + e)) : __ldg(g.pts + e);
+  return __ldg(g.pts + __ldg(g.cand + e));
 }
 
 __device__ __forceinline__ int point_item(float4 p) { return __float_as_int(p.w); }
-
-// The same for a grid whose entry form is known at compile time (kIdx: item
-// indices), for the per-entry loop of the one-thread pass.
-template <bool kIdx>
-__device__ __forceinline__ float4 grid_point_of(const GridView& g, int e) {
-  if constexpr (kIdx)
-    return __ldg(g.pts + __ldg(g.cand + e));
-  else
-    return __ldg(g.pts + e);
-}
 
 // min(dmax2, squared distances to the points of this lane's candidate list),
 // for the 32 lanes of a warp together (all call it): lists of at most thr
@@ -429,7 +419,6 @@ __device__ __forceinline__ float4 grid_point_of(const GridView& g, int e) {
 // the exact minimum over the list, whatever the split; a warp whose lists
 // differ widely in length (every kept point as the collision set) no longer
 // runs its longest list on one lane while the others idle.
-template <bool kIdx>
 __device__ __forceinline__ float warp_split_min(const GridView& g, int2 range, float px, float py,
                                                 float pz, float dmax2, int thr) {
   const int lane = threadIdx.x & 31;
@@ -437,7 +426,7 @@ __device__ __forceinline__ float warp_split_min(const GridView& g, int2 range, f
   float d2 = dmax2;
   if (!lng)
     for (int i = 0; i < range.y; ++i)
-      d2 = fminf(d2, dist2_to(grid_point_of<kIdx>(g, range.x + i), px, py, pz));
+      d2 = fminf(d2, dist2_to(grid_point(g, range.x + i), px, py, pz));
   unsigned pend = __ballot_sync(0xffffffffu, lng);
   while (pend) {
     const int L = __ffs(pend) - 1;
@@ -449,7 +438,7 @@ __device__ __forceinline__ float warp_split_min(const GridView& g, int2 range, f
     const float qz = __shfl_sync(0xffffffffu, pz, L);
     unsigned best = __float_as_uint(dmax2);
     for (int i = lane; i < n; i += 32) {
-      const float d = dist2_to(grid_point_of<kIdx>(g, first + i), qx, qy, qz);
+      const float d = dist2_to(grid_point(g, first + i), qx, qy, qz);
       if (d < dmax2) best = min(best, __float_as_uint(d));
     }
     best = __reduce_min_sync(0xffffffffu, best);
@@ -465,22 +454,15 @@ __device__ __forceinline__ float warp_split_min(const GridView& g, int2 range, f
 template <int kW = 4>
 __device__ __forceinline__ float scan_min(const GridView& g, int first, int n, float px, float py,
                                           float pz, float best) {
-  const uint32_t* E = g.cand ? g.cand + first : nullptr;
-  const float4* P = g.cand ? g.pts : g.pts + first;
+  const uint32_t* E = g.cand + first;
   for (int t = 0; t < n; t += kW) {
     float4 c[kW];
-    if (E) {
-      uint32_t id[kW];
-      id[0] = __ldg(E + t);
+    uint32_t id[kW];
+    id[0] = __ldg(E + t);
 #pragma unroll
-      for (int i = 1; i < kW; ++i) id[i] = t + i < n ? __ldg(E + t + i) : id[0];
+    for (int i = 1; i < kW; ++i) id[i] = t + i < n ? __ldg(E + t + i) : id[0];
 #pragma unroll
-      for (int i = 0; i < kW; ++i) c[i] = __ldg(P + id[i]);
-    } else {
-      c[0] = __ldg(P + t);
-#pragma unroll
-      for (int i = 1; i < kW; ++i) c[i] = t + i < n ? __ldg(P + t + i) : c[0];
-    }
+    for (int i = 0; i < kW; ++i) c[i] = __ldg(g.pts + id[i]);
     float m = dist2_to(c[0], px, py, pz);
 #pragma unroll
     for (int i = 1; i < kW; ++i) m = fminf(m, dist2_to(c[i], px, py, pz));

@@ -83,14 +83,24 @@ struct CandArgs {
   int* fill;           // G^3 + 1: fill cursors of the scatter pass; zeroed by the scan
   const int* local;    // tile-local exclusive prefix of the counts (scatter pass)
   const int* tile_off; // exclusive prefix of the tile totals (scatter pass)
-  // candidate entries (scatter pass), in one of two forms: item indices into
-  // pts, whose points the count pass stores (cand non-null), or the points
-  // themselves (cand4)
-  uint32_t* cand;
-  float4* pts;         // n_items: collision point of each item, minus p0 (w: the item index's bits)
-  float4* cand4;       // entries holding the points (w: the item index's bits)
+  uint32_t* cand;      // candidate entries (scatter pass): item indices into pts
+  float4* pts;         // n_items: collision point of each item, minus p0 (w: the item index's
+                       // bits; stored by the count pass)
   int* status;
   unsigned long long* reset_keys;  // non-null: the scatter pass empties each key it reads
+};
+
+// Pruning of the candidate lists.
+struct PruneArgs {
+  uint32_t* cand;          // entries, permuted within each list: the kept ones last
+  const float4* pts;       // collision point of each item
+  int2* range;             // {first entry, count} of each cell: of the kept ones afterwards
+  int items;               // collision items
+  int ncells;
+  int runs;                // runs of cells per unit (set by the launch)
+  const int* total;        // entries of all lists, or null; below min_total the lists stay whole
+  int min_total;
+  GridGeom grid;
 };
 
 struct GuideArgs {
@@ -116,8 +126,8 @@ struct GuideArgs {
 
 struct GridView {
   const int2* range;     // G^3 cell ranges into the candidate entries
-  const uint32_t* cand;  // entries as item indices into pts, grouped by cell; or null:
-  const float4* pts;     // the items' collision points (minus p0), or (cand null) the entries' own
+  const uint32_t* cand;  // entries, grouped by cell: item indices into pts
+  const float4* pts;     // the items' collision points (minus p0)
   int G;
   float origin, inv_h;
 };
@@ -202,6 +212,7 @@ __host__ __device__ constexpr size_t warm_words(int E, int T) {
 // ---------------------------------------------------------------------------
 constexpr int kBatchMax = 256;       // planners per batched call
 constexpr int kPartChunk = 1024;     // points per partition unit
+constexpr int kPruneCells = 256;     // cells per pruning block, at most
 
 enum BatchPrefix {
   kPrePoints = 0,  // partition units (kPartChunk points)
@@ -209,6 +220,7 @@ enum BatchPrefix {
   kPreCoarse,      // coarse cells (one warp each)
   kPreTiles,       // scan tiles
   kPreCells,       // grid cells (range of each) and, after them, raw-set keys to reset
+  kPrePrune,       // pruning units (kPruneCells cells)
   kPreRoll1,       // rollout units, one lane per sample, in order1
   kPreRoll4,       // rollout units, four lanes per sample, in order4
   kPreUpdate,      // (planner, instance) units of the update
@@ -250,6 +262,7 @@ cudaError_t launch_batch_partition(const BatchView& v, int blocks, cudaStream_t 
 cudaError_t launch_batch_count(const BatchView& v, int blocks, cudaStream_t s);
 cudaError_t launch_batch_scan(const BatchView& v, int blocks, cudaStream_t s);
 cudaError_t launch_batch_scatter(const BatchView& v, int blocks, cudaStream_t s);
+cudaError_t launch_batch_prune(const BatchView& v, int blocks, cudaStream_t s);
 // lanes 1 or 4; dynamic: take units from the work queue, else stride by the grid;
 // six: the one-lane kernel compiled for six resident CTAs per SM (fewer
 // registers) instead of five; samples_per_cta: the one-lane pass's CTA size
@@ -258,10 +271,10 @@ cudaError_t launch_batch_rollout(const BatchView& v, int lanes, int it, int bloc
                                  int six, int samples_per_cta, cudaStream_t s);
 cudaError_t launch_batch_update(const BatchView& v, int it, int blocks, cudaStream_t s);
 
-// Resident CTAs per SM: {partition, count, scan, scatter} and {rollout with one
+// Resident CTAs per SM: {partition, count, scan, scatter, prune} and {rollout with one
 // lane per sample, with four, update, rollout with one lane compiled for six,
 // one lane with 64 samples per CTA, one lane with 256}.
-cudaError_t batch_grid_occupancy(int out[4]);
+cudaError_t batch_grid_occupancy(int out[5]);
 cudaError_t batch_rollout_occupancy(int out[6], int T_max);
 
 // t: the edge tables in device memory
@@ -280,6 +293,9 @@ cudaError_t launch_grid_scan(int* count, int* fill, int* local, int* tile_sum, i
 // totals of the scan launch (and written to tile_off)
 cudaError_t launch_grid_scatter(const CandArgs& ca, int2* range, int ncells, const int* tile_sum,
                                 int* tile_off, int ntiles, cudaStream_t s);
+// the lists pruned to the entries that can be a query's nearest, the ranges with them
+cudaError_t launch_grid_prune(PruneArgs a, cudaStream_t s);
+cudaError_t prune_attributes();  // its shared-memory limit (set by split_attributes)
 // S(1) of n noise-free rollouts of instance `instance` and their gradients.
 struct CostGradArgs {
   UpdateArgs ctx;          // x0, dynamics, costs, grid, guides, T of the last step
@@ -341,6 +357,7 @@ enum CheckBit : int {
   kChkQuery = 1 << 11,       // split pass / Stage II: query slot or item outside its list
   kChkPartial = 1 << 12,     // partial row or sample outside the instance's block
   kChkAccum = 1 << 13,       // accumulation ring slot
+  kChkPrune = 1 << 14,       // list pruning: entry, item or scratch slot outside its array
 };
 #ifdef AERO_CHECKED
 static __device__ int g_check_word;

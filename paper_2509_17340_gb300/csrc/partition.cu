@@ -8,6 +8,7 @@
 // so they are a defined function of the binary32 inputs.
 #include <cfloat>
 #include <cstdint>
+#include <type_traits>
 
 #include "device.cuh"
 #include "internal.h"
@@ -329,12 +330,11 @@ __global__ void __launch_bounds__(256) k_partition(PartitionArgs a, const PartTa
 // K2a / K2d: candidate lists.  For every collision point p (item i), every
 // cell whose box is closer to p than `reach` gets p: the count pass adds to
 // the cell's counter, the scatter pass writes the entry at start(cell) + its
-// fill ticket.  An entry is either i (4 bytes; the count pass stores p at
-// pts[i], and the points, far fewer than the entries, stay in L1) or p itself
-// (16 bytes, one load fewer per entry read).  Either way a point carries its
-// item index in w (bits of an int), so that ties between equidistant points
-// are broken by item, the collision set's order, whatever the order of the
-// entries within a cell, which depends on the atomics.
+// fill ticket.  An entry is i (the
+// count pass stores p at pts[i]; the points, far fewer than the entries, stay in
+// L1).  A point carries its item index in w (bits of an int), so that ties between
+// equidistant points are broken by item, the collision set's order, whatever the
+// order of the entries within a cell, which depends on the atomics.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ bool cand_item(const CandArgs& a, int64_t it, float& px, float& py,
                                           float& pz) {
@@ -360,9 +360,7 @@ __device__ __forceinline__ float gap2(float v, float lo, float h) {
 }
 
 // One warp per collision item; its lanes share the item's block of cells.
-// kIdx: the entries are item indices (a single planner's step), else points
-// (batched steps); the form is fixed per launch, so it is a template argument.
-template <bool kScatter, bool kIdx>
+template <bool kScatter>
 __device__ __forceinline__ void cand_task(const CandArgs& a, int64_t it, int lane) {
   const GridGeom& g = a.grid;
   const float r2 = g.reach * g.reach;
@@ -373,7 +371,7 @@ __device__ __forceinline__ void cand_task(const CandArgs& a, int64_t it, int lan
     __syncwarp();
     if (lane == 0) a.reset_keys[it] = kEmpty;
   }
-  if constexpr (!kScatter && kIdx) {
+  if constexpr (!kScatter) {
     if (lane == 0) a.pts[it] = make_float4(px, py, pz, __int_as_float((int)it));
   }
   const int x0 = max(__float2int_rd((px - g.reach - g.origin) * g.inv_h), 0);
@@ -427,10 +425,7 @@ __device__ __forceinline__ void cand_task(const CandArgs& a, int64_t it, int lan
         if (c[b] < 0) continue;
         const int pos = base[b] + ticket[b];
         if (pos < g.cap) {
-          if constexpr (kIdx)
-            a.cand[pos] = (uint32_t)it;
-          else
-            a.cand4[pos] = make_float4(px, py, pz, __int_as_float((int)it));
+          a.cand[pos] = (uint32_t)it;
         } else {
           atomicOr(a.status, 2);
         }
@@ -445,7 +440,7 @@ __device__ void cand_pass(const CandArgs& a, int block, int nblocks) {
   const int lane = threadIdx.x & 31;
   const int64_t warps = (int64_t)nblocks * (blockDim.x >> 5);
   for (int64_t it = ((int64_t)block * blockDim.x + threadIdx.x) >> 5; it < a.n_items; it += warps)
-    cand_task<kScatter, true>(a, it, lane);
+    cand_task<kScatter>(a, it, lane);
 }
 
 // ---------------------------------------------------------------------------
@@ -749,6 +744,276 @@ __global__ void __launch_bounds__(256) k_grid_scatter(CandArgs ca, int scatter_b
     range_cell(ca.local, s_off, ca.grid.cap, range, c);
 }
 
+// ---------------------------------------------------------------------------
+// K2e: pruned lists.  Entry p of a cell's list can be left out of the cell's
+// queries when another entry q is nearer to every point x of the cell's box:
+// |x - q|^2 - |x - p|^2 is linear in x, so its maximum over the box (centre m, half
+// edges b) is |q - m|^2 - |p - m|^2 + 2 b |p - q|_1, and p is dominated when that
+// is below a margin that covers the rounding of this test, of the queries' cells
+// and of their distances.  A dominated p is then never the nearest point in
+// binary32 either, nor equidistant with it, so the queries' minima, nearest points
+// and ties are those of the whole list, bit for bit.  Dominance is a strict partial
+// order: whatever dominates p is itself kept or dominated by something kept.
+// The list is permuted, the kept entries last, and the cell's range covers those.
+//
+// A list of 10 to 500 entries keeps a quarter to a tenth of them (the others lie
+// beside and behind the nearest ones), and Stage I's time is in scanning the longest
+// list of each warp's queries: with every kept point (178,000) 2.99 -> 0.95 ms, large
+// clutter 344 -> 277 us, flight cycle (split pass) 136 -> 67, a dense map 108 -> 48,
+// 64 batched planners 1055 -> 823, for 318, 36, 50, 70 and 221 us of pruning.
+// ---------------------------------------------------------------------------
+constexpr int kPruneMin = 5;        // shorter lists stay whole
+constexpr int kPruneThreads = 256;
+constexpr int kPruneHead = 128;     // entries of a list that the seeds are taken from
+constexpr int kPruneKeep = 640;     // kept entries of a list in shared memory
+constexpr int kPruneSeeds = 9;
+constexpr int kPruneRun = 4;        // consecutive cells of a block
+
+// The lists of a block's cells by length: up to 8 entries (four lists per warp), up
+// to 16 (two), and longer (one).
+enum PruneClass { kPrune8 = 0, kPrune16, kPruneWarp, kPruneClasses };
+
+struct PruneSmem {
+  struct {
+    float4 p[kPruneHead];    // the head's points, w: squared distance to the box centre
+    uint32_t tag[kPruneHead];
+    uint32_t keep[kPruneKeep];
+    float4 seed[kPruneSeeds];
+  } w[kPruneThreads / 32];
+  int2 range[kPruneCells];  // the lists in the order of their classes
+  int cell[kPruneCells];
+  int n[kPruneClasses], at[kPruneClasses], next[kPruneClasses];
+};
+
+// A list's box: twice the half edge (with the rounding of the queries' cells and of
+// the centre, below 1e-6 of the grid's extent) and the margin, 1e-5 of the largest
+// squared distance compared, whose own rounding is below 1e-6 of it.
+struct PruneBox {
+  float3 m;
+  float b2, margin;
+};
+
+__device__ __forceinline__ PruneBox prune_box(const GridGeom& g, int c) {
+  PruneBox b;
+  b.m = make_float3(g.origin + (c % g.G + 0.5f) * g.h, g.origin + (c / g.G % g.G + 0.5f) * g.h,
+                    g.origin + (c / (g.G * g.G) + 0.5f) * g.h);
+  b.b2 = g.h - 8e-6f * g.origin;
+  b.margin = 1e-5f * (g.reach + g.h) * (g.reach + g.h);
+  return b;
+}
+
+__device__ __forceinline__ bool dominated(float4 q, float4 p, const PruneBox& b) {
+  return q.w - p.w + b.b2 * (fabsf(p.x - q.x) + fabsf(p.y - q.y) + fabsf(p.z - q.z)) < -b.margin;
+}
+
+// Entry i's point; `tag`: the entry.  Through L2: a line of the array also holds
+// other lists' entries, which other SMs permute meanwhile, and the queries read
+// the same lines next.  (Bounds compared in every build: nothing that an earlier
+// pass left wrong makes this one leave the arrays.)
+__device__ __forceinline__ float4 prune_load(const PruneArgs& a, int i, const PruneBox& b, uint32_t& tag) {
+  tag = 0;
+  if ((unsigned)i >= (unsigned)a.grid.cap) return make_float4(0.f, 0.f, 0.f, INFINITY);
+  tag = __ldcg(a.cand + i);
+  if (!AERO_CHECK(tag < (uint32_t)a.items, kChkPrune) || tag >= (uint32_t)a.items)
+    return make_float4(0.f, 0.f, 0.f, INFINITY);
+  const float4 p = __ldg(a.pts + tag);
+  const float x = p.x - b.m.x, y = p.y - b.m.y, z = p.z - b.m.z;
+  return make_float4(p.x, p.y, p.z, x * x + y * y + z * z);
+}
+
+__device__ __forceinline__ void prune_store(const PruneArgs& a, int i, uint32_t tag) {
+  if (AERO_CHECK((unsigned)i < (unsigned)a.grid.cap, kChkPrune) && (unsigned)i < (unsigned)a.grid.cap)
+    __stcg(a.cand + i, tag);
+}
+
+// The seeds of a list: the entries nearest to the box's centre and to its eight
+// corners.  Any entries would do (a wrong choice only leaves more entries in), so the
+// nearest is found by the upper bits of the squared distance with the entry's number
+// within the lane below them.  What nine seeds keep is within a few percent of all
+// that a comparison of every pair keeps where lists are short (P_f) and half as
+// much again on dense surfaces.
+__device__ __forceinline__ void seed_keys(uint32_t* key, float4 p, const PruneBox& b, uint32_t mask, uint32_t id) {
+  const float x = (p.x - b.m.x) * b.b2, y = (p.y - b.m.y) * b.b2, z = (p.z - b.m.z) * b.b2;
+  auto take = [&](int k, float d) {
+    key[k] = min(key[k], (__float_as_uint(fmaxf(d, 0.0f)) & ~mask) | id);
+  };
+  take(0, p.w);
+  const float w = p.w + 0.75f * b.b2 * b.b2;  // to a corner: |p - m|^2 -+ x -+ y -+ z + 3 (b2 / 2)^2
+  const float a = w - x - y, c = w - x + y, d = w + x - y, e = w + x + y;
+  take(1, a - z);
+  take(2, a + z);
+  take(3, c - z);
+  take(4, c + z);
+  take(5, d - z);
+  take(6, d + z);
+  take(7, e - z);
+  take(8, e + z);
+}
+
+// Lists of at most W entries, one per group of W lanes, each entry compared with
+// each.  Returns the range of the kept ones.
+template <int W>
+__device__ __forceinline__ int2 prune_group(const PruneArgs& a, int2 r, const PruneBox& b, int lane) {
+  const int i = lane % W;
+  float4 p = make_float4(0.f, 0.f, 0.f, INFINITY);
+  uint32_t tag = 0;
+  const bool in = i < r.y;
+  if (in) p = prune_load(a, r.x + i, b, tag);
+  bool ok = in;
+#pragma unroll
+  for (int j = 0; j < W; ++j) {
+    const float4 q = make_float4(__shfl_sync(0xffffffffu, p.x, j, W), __shfl_sync(0xffffffffu, p.y, j, W),
+                                 __shfl_sync(0xffffffffu, p.z, j, W), __shfl_sync(0xffffffffu, p.w, j, W));
+    if (dominated(q, p, b)) ok = false;
+  }
+  const int g = lane - i;
+  const unsigned mask = (1u << W) - 1u, below = (1u << i) - 1u;
+  const unsigned kb = __ballot_sync(0xffffffffu, ok) >> g & mask;
+  const unsigned db = __ballot_sync(0xffffffffu, in && !ok) >> g & mask;
+  const int kept = __popc(kb);
+  if (db != 0) {  // (a list that stays whole is not rewritten)
+    if (ok) prune_store(a, r.x + r.y - 1 - __popc(kb & below), tag);
+    else if (in) prune_store(a, r.x + __popc(db & below), tag);
+  }
+  return make_int2(r.x + r.y - kept, kept);
+}
+
+// A longer list by one warp: the seeds from its first entries, then every entry
+// against them, 32 at a time (the loads of four turns together); the entries left out
+// move to the front of the list, over places already read, the kept ones wait in
+// shared memory.  A list that keeps more than fits ends there, the rest of it whole.
+// The launch is bound by the latency of these loads and by fetching its code, which
+// a warp runs a few times only: one list per warp rather than per block, and short
+// loops rather than unrolled registers.
+__device__ __forceinline__ int2 prune_warp(const PruneArgs& a, PruneSmem& sm, int2 r, const PruneBox& b, int wid,
+                                           int lane) {
+  auto& w = sm.w[wid];
+  const int n = r.y, head = min(n, kPruneHead);
+  __syncwarp();  // the scratch is free
+#pragma unroll 4
+  for (int i = lane; i < head; i += 32) {
+    uint32_t tag;
+    w.p[i] = prune_load(a, r.x + i, b, tag);
+    w.tag[i] = tag;
+  }
+  uint32_t key[kPruneSeeds];
+#pragma unroll
+  for (int k = 0; k < kPruneSeeds; ++k) key[k] = 0xffffffffu;
+#pragma unroll 1
+  for (int i = lane; i < head; i += 32) seed_keys(key, w.p[i], b, 3u, i >> 5);
+#pragma unroll
+  for (int k = 0; k < kPruneSeeds; ++k) {
+    const uint32_t best = __reduce_min_sync(0xffffffffu, key[k]);
+    if (key[k] == best) w.seed[k] = w.p[((best & 3u) << 5) + lane];  // (of several equal ones any)
+  }
+  __syncwarp();
+  int kept = 0, dead = 0, i0 = 0;
+  bool full = false;
+  const unsigned below = (1u << lane) - 1u;
+#pragma unroll 1
+  for (; i0 < n && !full; i0 += kPruneHead) {
+    if (i0 > 0) {
+      __syncwarp();
+#pragma unroll
+      for (int s = 0; s < kPruneHead / 32; ++s) {
+        const int i = 32 * s + lane;
+        uint32_t tag = 0;
+        if (i0 + i < n) w.p[i] = prune_load(a, r.x + i0 + i, b, tag);
+        w.tag[i] = tag;
+      }
+      __syncwarp();
+    }
+    full = kept + kPruneHead > kPruneKeep;  // the turn's kept ones might not fit
+    if (full) break;
+#pragma unroll 1
+    for (int s = lane; s < kPruneHead && i0 + s - lane < n; s += 32) {
+      const bool in = i0 + s < n;
+      const float4 p = w.p[s];
+      bool k = in;
+#pragma unroll 3
+      for (int j = 0; j < kPruneSeeds; ++j)
+        if (dominated(w.seed[j], p, b)) k = false;
+      const unsigned kb = __ballot_sync(0xffffffffu, k), db = __ballot_sync(0xffffffffu, in && !k);
+      const int at = kept + __popc(kb & below);
+      if (k && AERO_CHECK(at < kPruneKeep, kChkPrune)) w.keep[at] = w.tag[s];
+      if (in && !k) prune_store(a, r.x + dead + __popc(db & below), w.tag[s]);
+      kept += __popc(kb);
+      dead += __popc(db);
+    }
+  }
+  __syncwarp();
+#pragma unroll 1
+  for (int i = lane; i < kept; i += 32) prune_store(a, r.x + dead + i, w.keep[i]);
+  return make_int2(r.x + dead, n - dead);
+}
+
+// The cell of this thread in unit `unit` of `units`: a.runs runs of kPruneRun cells,
+// spread over the whole grid, for the long lists lie together (near the start, on
+// dense surfaces).  -1: none.
+__device__ __forceinline__ int prune_cell_of(int runs, int ncells, int unit, int units) {
+  const int tid = threadIdx.x;
+  const int c = ((tid / kPruneRun) * units + unit) * kPruneRun + tid % kPruneRun;
+  return tid < runs * kPruneRun && c < ncells ? c : -1;
+}
+
+// The block prunes its threads' lists (cell c, range r; r.y = 0: none).
+__device__ void prune_cells(const PruneArgs& a, PruneSmem& sm, int c, int2 r) {
+  const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+  if (tid < kPruneClasses) sm.n[tid] = sm.next[tid] = 0;
+  __syncthreads();
+  int cls = -1, slot = 0;
+  if (r.y >= kPruneMin) {
+    cls = r.y <= 8 ? kPrune8 : r.y <= 16 ? kPrune16 : kPruneWarp;
+    slot = atomicAdd(&sm.n[cls], 1);
+  }
+  __syncthreads();
+  if (tid < kPruneClasses) {
+    int at = 0;
+    for (int k = 0; k < tid; ++k) at += sm.n[k];
+    sm.at[tid] = at;
+  }
+  __syncthreads();
+  if (cls >= 0 && AERO_CHECK(sm.at[cls] + slot < kPruneCells, kChkPrune)) {
+    sm.range[sm.at[cls] + slot] = r;
+    sm.cell[sm.at[cls] + slot] = c;
+  }
+  __syncthreads();
+  // the warps take the lists, the longest class first
+  auto take = [&](int k, int lists) {
+    int q = 0;
+    if (lane == 0) q = atomicAdd(&sm.next[k], lists);
+    return __shfl_sync(0xffffffffu, q, 0);
+  };
+  for (;;) {
+    const int q = take(kPruneWarp, 1);
+    if (q >= sm.n[kPruneWarp]) break;
+    const int at = sm.at[kPruneWarp] + q;
+    r = prune_warp(a, sm, sm.range[at], prune_box(a.grid, sm.cell[at]), wid, lane);
+    if (lane == 0) a.range[sm.cell[at]] = r;
+  }
+  auto groups = [&](auto width, int k) {
+    constexpr int W = decltype(width)::value;
+    for (;;) {
+      const int q = take(k, 32 / W);
+      if (q >= sm.n[k]) break;
+      const bool on = q + lane / W < sm.n[k];
+      const int at = sm.at[k] + q + (on ? lane / W : 0), cell = sm.cell[at];
+      const int2 r1 = prune_group<W>(a, on ? sm.range[at] : make_int2(0, 0), prune_box(a.grid, cell), lane);
+      if (on && lane % W == 0) a.range[cell] = r1;
+    }
+  };
+  groups(std::integral_constant<int, 16>(), kPrune16);
+  groups(std::integral_constant<int, 8>(), kPrune8);
+}
+
+__global__ void __launch_bounds__(kPruneThreads) k_grid_prune(PruneArgs a) {
+  pdl_start();
+  if (a.total && __ldg(a.total) < a.min_total) return;
+  extern __shared__ __align__(16) unsigned char prune_smem[];
+  const int c = prune_cell_of(a.runs, a.ncells, blockIdx.x, gridDim.x);
+  prune_cells(a, *reinterpret_cast<PruneSmem*>(prune_smem), c, c >= 0 ? a.range[c] : make_int2(0, 0));
+}
+
 __global__ void k_philox(uint32_t k0, uint32_t k1, uint32_t c1, uint32_t c2, uint32_t c3,
                          int64_t n, uint4* out) {
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -822,7 +1087,7 @@ __device__ __forceinline__ void cand_tasks(const BatchView& v, const long long* 
         while (t >= s_pi[it + 1]) ++it;
         a = v.items[it].ca;
       }
-      cand_task<kScatter, false>(a, t - s_pi[it], lane);
+      cand_task<kScatter>(a, t - s_pi[it], lane);
     }
   }
 }
@@ -901,6 +1166,39 @@ __global__ void __launch_bounds__(256) k_b_scatter(BatchView v) {
   }
 }
 
+// Units (planner, kPruneCells cells).
+__global__ void __launch_bounds__(kPruneThreads) k_b_prune(BatchView v) {
+  pdl_start();
+  extern __shared__ __align__(16) unsigned char prune_smem[];
+  __shared__ long long s_pp[kBatchMax + 1];
+  const int n = v.n;
+  load_prefix(s_pp, v.pre + kPrePrune * (n + 1), n);
+  __syncthreads();
+  const long long total = s_pp[n];
+  int it = 0, c = -1;
+  int2 r = make_int2(0, 0);
+  auto fetch = [&](long long u) {  // unit u's planner, and this thread's cell and range in it
+    c = -1;
+    r = make_int2(0, 0);
+    if (u >= total) return;
+    it = find_unit(s_pp, n, u);
+    const BatchItem* bi = v.items + it;
+    c = prune_cell_of(kPruneCells / kPruneRun, bi->gcells, (int)(u - s_pp[it]), (int)(s_pp[it + 1] - s_pp[it]));
+    if (c >= 0) r = bi->range[c];
+  };
+  fetch(blockIdx.x);
+  for (long long u = blockIdx.x; u < total; u += gridDim.x) {
+    const BatchItem* bi = v.items + it;
+    const int cu = c;
+    const int2 ru = r;
+    fetch(u + gridDim.x);  // the next unit's ranges are on their way meanwhile
+    const PruneArgs a{bi->ca.cand, bi->ca.pts, bi->range, (int)bi->ca.n_items, bi->gcells,
+                      kPruneCells / kPruneRun, nullptr, 0, bi->ca.grid};
+    prune_cells(a, *reinterpret_cast<PruneSmem*>(prune_smem), cu, ru);
+    __syncthreads();  // the unit's shared memory is free again
+  }
+}
+
 int blocks_for(int64_t n, int threads, int cap) {
   int64_t b = (n + threads - 1) / threads;
   if (b < 1) b = 1;
@@ -949,13 +1247,33 @@ cudaError_t launch_grid_scatter(const CandArgs& ca, int2* range, int ncells, con
                   scatter_blocks, range, ncells, tile_sum, tile_off, ntiles);
 }
 
-cudaError_t batch_grid_occupancy(int out[4]) {
-  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out + 0, k_b_partition, 256, 0);
+cudaError_t launch_grid_prune(PruneArgs a, cudaStream_t s) {
+  // the largest grid in blocks of 256 cells, a smaller one in smaller blocks, at
+  // least about eight per SM
+  a.runs = kPruneCells / kPruneRun;
+  while (a.runs > 8 && a.ncells < 8 * device_sms() * a.runs * kPruneRun) a.runs /= 2;
+  const int cells = a.runs * kPruneRun, units = (a.ncells + cells - 1) / cells;
+  return launch_ks(k_grid_prune, dim3(units), dim3(kPruneThreads), sizeof(PruneSmem),
+                   s, true, a);
+}
+
+cudaError_t prune_attributes() {
+  const cudaError_t e =
+      cudaFuncSetAttribute(k_grid_prune, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PruneSmem));
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(k_b_prune, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PruneSmem));
+}
+
+cudaError_t batch_grid_occupancy(int out[5]) {
+  cudaError_t e = prune_attributes();
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out + 0, k_b_partition, 256, 0);
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out + 1, k_b_count, 256, 0);
   if (e == cudaSuccess)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out + 2, k_b_scan, kScanThreads, 0);
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out + 3, k_b_scatter, 256, 0);
-  for (int i = 0; i < 4; ++i)
+  if (e == cudaSuccess)
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out + 4, k_b_prune, kPruneThreads, sizeof(PruneSmem));
+  for (int i = 0; i < 5; ++i)
     if (out[i] < 1) out[i] = 1;
   return e;
 }
@@ -975,6 +1293,10 @@ cudaError_t launch_batch_scan(const BatchView& v, int blocks, cudaStream_t s) {
 
 cudaError_t launch_batch_scatter(const BatchView& v, int blocks, cudaStream_t s) {
   return launch_k(k_b_scatter, dim3(blocks), dim3(256), s, true, v);
+}
+
+cudaError_t launch_batch_prune(const BatchView& v, int blocks, cudaStream_t s) {
+  return launch_ks(k_b_prune, dim3(blocks), dim3(kPruneThreads), sizeof(PruneSmem), s, true, v);
 }
 
 cudaError_t launch_philox(uint32_t k0, uint32_t k1, uint32_t c1, uint32_t c2, uint32_t c3,

@@ -37,12 +37,12 @@ struct CostSum {
 
 // Samples [b * kNT, (b + 1) * kNT) of instance e, one per thread (kNT: the
 // CTA's threads, a multiple of 32); ctr3: the noise counter's last word,
-// (step_id << 8) | iteration.  kIdx: the grid's candidate entries are item
-// indices (a single planner's step), else points (batched steps).
+// (step_id << 8) | iteration.  kParams: the arguments are
+// kernel parameters (a single planner's step), else in shared memory.
 // kWarpLists: long candidate lists scanned by the whole warp (warp_split_min,
-// lists longer than a.list_thr), for the every-point collision set; the
-// short lists of P_f keep the per-lane scan, compiled without that path.
-template <bool kIdx, int kNT = NT, bool kWarpLists = false, bool kRestForm = kIdx && !kWarpLists>
+// lists longer than a.list_thr), for every-point collision sets whose lists are not
+// pruned; the others keep the per-lane scan, compiled without that path.
+template <bool kParams, int kNT = NT, bool kWarpLists = false, bool kRestForm = kParams && !kWarpLists>
 __device__ __forceinline__ void rollout_unit(const RolloutArgs& a, int e, int b, uint32_t ctr3) {
   constexpr int kNW = kNT / 32;
   constexpr int kSW = kNT > kMaxT ? kNT : kMaxT;
@@ -67,7 +67,7 @@ __device__ __forceinline__ void rollout_unit(const RolloutArgs& a, int e, int b,
   const float dmax2 = cp.d_max * cp.d_max;
   // kRestForm: the at-rest goal term compiled in.  Left out of the batched
   // passes built for 80 registers (the test's registers made them spill) and
-  // of the every-point instance (17% slower with it)
+  // of the warp-list instance (17% slower with it)
   const bool at_rest = kRestForm && goal_at_rest(cp);
   const int dbg = (active && k < a.dbg_D) ? (e * a.dbg_D + k) : -1;
   const float4 sigma = make_float4(a.sigma[0], a.sigma[1], a.sigma[2], a.sigma[3]);
@@ -93,7 +93,7 @@ __device__ __forceinline__ void rollout_unit(const RolloutArgs& a, int e, int b,
   // are read as constant operands; the batched kernels' are in shared memory,
   // where recomputing the schedule is cheaper than reading it
   auto noise = [&](uint32_t kk, uint32_t j) {
-    if constexpr (kIdx)
+    if constexpr (kParams)
       return noise_delta_rk(kk, j, e, ctr3, a.rk, sigma);
     else
       return noise_delta(kk, j, e, ctr3, a.key0, a.key1, sigma);
@@ -131,7 +131,7 @@ __device__ __forceinline__ void rollout_unit(const RolloutArgs& a, int e, int b,
   // from one step to the next alternates between two register sets instead
   // of being copied (the batched kernels, with their arguments in shared
   // memory, would spill)
-  constexpr int kUnroll = kIdx ? 2 : 1;
+  constexpr int kUnroll = kParams ? 2 : 1;
 #pragma unroll kUnroll
   for (int j = 1; j <= T; ++j) {
     const int2 range_j = range;
@@ -147,11 +147,11 @@ __device__ __forceinline__ void rollout_unit(const RolloutArgs& a, int e, int b,
     // that instance ran 2.85 instead of 3.33 ms at 200,000 kept points)
     float d2 = dmax2;
     if (kWarpLists && a.list_thr > 0) {
-      d2 = warp_split_min<kIdx>(a.grid, active ? range_j : make_int2(0, 0), x.p[0], x.p[1], x.p[2],
-                                dmax2, a.list_thr);
+      d2 = warp_split_min(a.grid, active ? range_j : make_int2(0, 0), x.p[0], x.p[1], x.p[2], dmax2,
+                          a.list_thr);
     } else {
       for (int i = 0; i < range_j.y; ++i)
-        d2 = fminf(d2, dist2_to(grid_point_of<kIdx>(a.grid, range_j.x + i), x.p[0], x.p[1], x.p[2]));
+        d2 = fminf(d2, dist2_to(grid_point(a.grid, range_j.x + i), x.p[0], x.p[1], x.p[2]));
     }
     // state terms at x_j against the guide at t = j dt
     const float gx = s_gd[3 * (j - 1)], gy = s_gd[3 * (j - 1) + 1], gz = s_gd[3 * (j - 1) + 2];
@@ -1098,6 +1098,7 @@ cudaError_t split_attributes() {
                              (int)update_smem_bytes(kMaxT, ST / 32, true));
   if (r == cudaSuccess)
     r = cudaFuncSetAttribute(k_b_update, cudaFuncAttributeMaxDynamicSharedMemorySize, refine);
+  if (r == cudaSuccess) r = prune_attributes();
   if (cached) done[dev].store(r == cudaSuccess ? 1 : (int)r + 2);
   return r;
 }
