@@ -904,7 +904,10 @@ __device__ __forceinline__ int2 prune_warp(const PruneArgs& a, PruneSmem& sm, in
 #pragma unroll
   for (int k = 0; k < kPruneSeeds; ++k) {
     const uint32_t best = __reduce_min_sync(0xffffffffu, key[k]);
-    if (key[k] == best) w.seed[k] = w.p[((best & 3u) << 5) + lane];  // (of several equal ones any)
+    // of several equal ones the lowest lane's, by that lane alone: stores of four words
+    // by several lanes to one place may leave words of different entries, no entry's point
+    const unsigned equal = __ballot_sync(0xffffffffu, key[k] == best);
+    if (lane == __ffs(equal) - 1) w.seed[k] = w.p[((best & 3u) << 5) + lane];
   }
   __syncwarp();
   int kept = 0, dead = 0, i0 = 0;
