@@ -196,11 +196,16 @@ struct UpdateArgs {
                            // ticket}, both reset by its last CTA; or null
 };
 
-// One region of the warm-up scratch for E instances of horizon T (floats):
-// nominals E x T x 4, Stage II states (T + 1) x 10, candidate costs E, best
+// One region of the warm-up scratch for E instances of horizon T (floats): nominals
+// E x T x 4, one instance's Stage II states (T + 1) x 10, candidate costs E, best
 // sequence T x 4, then three words (best index, ticket, status).
+__host__ __device__ constexpr size_t warm_states_at(int E, int T) { return (size_t)E * T * 4; }
+__host__ __device__ constexpr size_t warm_cand_at(int E, int T) {
+  return warm_states_at(E, T) + (size_t)(T + 1) * 10;
+}
+__host__ __device__ constexpr size_t warm_best_at(int E, int T) { return warm_cand_at(E, T) + E; }
 __host__ __device__ constexpr size_t warm_words(int E, int T) {
-  return (size_t)E * T * 4 + (size_t)(T + 1) * 10 + E + (size_t)T * 4 + 3;
+  return warm_best_at(E, T) + (size_t)T * 4 + 3;
 }
 
 // ---------------------------------------------------------------------------

@@ -853,14 +853,38 @@ __global__ void __launch_bounds__(NT, 6) k_rollout(RolloutArgs a) {
 // critical path; the warm-up run's results are discarded.  It may read
 // partials that other CTAs are writing: every access of the update stays in
 // bounds whatever the values read.  Every thread of the CTA calls it.
+//
+// The region holds the Stage II states of instance e alone, where the update writes
+// those of instance e at e (T + 1) 10 from a.stage2_x: from where that pointer starts
+// (in region 0 or later: a region is longer than an instance's states).
+__host__ __device__ constexpr size_t warm_stage2_from(int E, int T, int e) {
+  return (size_t)e * warm_words(E, T) + warm_states_at(E, T) - (size_t)e * (T + 1) * 10;
+}
+
+// What the update of instance e reads and writes through these pointers lies in its parts
+// of region e (the offsets are linear in e: the first and the last instance).
+constexpr bool warm_regions_hold() {
+  for (int E = 1; E <= kMaxE; ++E)
+    for (int T = 1; T <= kMaxT; ++T)
+      for (int e = 0; e < E; e += E > 1 ? E - 1 : 1) {
+        const size_t base = (size_t)e * warm_words(E, T);
+        const size_t x = warm_stage2_from(E, T, e) + (size_t)e * (T + 1) * 10;
+        if (base + (size_t)(e + 1) * T * 4 > base + warm_states_at(E, T)) return false;
+        if (x < base + warm_states_at(E, T) || x + (size_t)(T + 1) * 10 > base + warm_cand_at(E, T)) return false;
+        if (warm_best_at(E, T) + (size_t)T * 4 + 3 > warm_words(E, T)) return false;
+      }
+  return true;
+}
+static_assert(warm_regions_hold(), "every warm-up run stays in its region");
+
 __device__ __forceinline__ void warm_setup(UpdateArgs* s_ua, const UpdateArgs& ua, int e) {
   const int E = ua.E, T = ua.T;
   float* const sc = ua.warm + (size_t)e * warm_words(E, T);
   if (threadIdx.x == 0) {
     s_ua->u_nom = sc;
-    s_ua->stage2_x = sc + (size_t)E * T * 4;
-    s_ua->cand = s_ua->stage2_x + (size_t)(T + 1) * 10;
-    s_ua->u_best = s_ua->cand + E;
+    s_ua->stage2_x = ua.warm + warm_stage2_from(E, T, e);
+    s_ua->cand = sc + warm_cand_at(E, T);
+    s_ua->u_best = sc + warm_best_at(E, T);
     s_ua->best_idx = reinterpret_cast<int*>(s_ua->u_best + (size_t)T * 4);
     s_ua->counter = reinterpret_cast<unsigned int*>(s_ua->best_idx + 1);
     s_ua->status = reinterpret_cast<int*>(s_ua->counter + 1);
