@@ -145,6 +145,7 @@ struct aero_planner {
   unsigned int* counter = nullptr;
   int* status = nullptr;
   float* warm = nullptr;      // warm-up scratch: E_max regions of warm_words(E_max, T_max)
+  WarmGrid* warm_grid = nullptr;  // the grid that the update launch's warm-up runs query
   float* dbg_u = nullptr;
   float* dbg_x = nullptr;
   float* dbg_d = nullptr;
@@ -337,7 +338,8 @@ void free_all(aero_planner* pl) {
                   pl->cand,     pl->cand_pts,   pl->grid_range, pl->partials,
                   pl->sample_costs, pl->stage2_x, pl->counter,   pl->status,   pl->dbg_u,
                   pl->dbg_x,    pl->dbg_d,      pl->stage_cloud,      pl->stage_out,
-                  pl->dbg_pre,      pl->part_counts,  pl->d_tab,  pl->warm};
+                  pl->dbg_pre,      pl->part_counts,  pl->d_tab,  pl->warm,
+                  pl->warm_grid};
   for (void* q : ptrs) dev_free(q);
   host_free(pl->h_out);
 }
@@ -595,6 +597,7 @@ void make_step_args(aero_planner* pl, const aero_state_t* x0, const float* cloud
   ua.inst_counter = pl->counter + 3;
   ua.status = pl->status;
   ua.warm = pl->warm;
+  ua.warm_grid = pl->warm_grid;
   ua.done = pl->warm != nullptr ? pl->counter + kDoneWord : nullptr;
   ra.done = ua.done;
 }
@@ -863,7 +866,10 @@ int create_planner(const aero_limits_t* limits, aero_planner_t** out, bool batch
   chk(alloc(&pl->stage2_x, (size_t)L.E_max * (L.T_max + 1) * 10));
   chk(alloc(&pl->counter, kCounterWords));
   chk(alloc(&pl->status, 1));
-  if (!batch_slot) chk(alloc(&pl->warm, (size_t)L.E_max * warm_words(L.E_max, L.T_max)));
+  if (!batch_slot) {
+    chk(alloc(&pl->warm, (size_t)L.E_max * warm_words(L.E_max, L.T_max)));
+    chk(alloc(&pl->warm_grid, 1));
+  }
   chk(alloc(&pl->dbg_u, (size_t)L.E_max * D * L.T_max * 4));
   chk(alloc(&pl->dbg_x, (size_t)L.E_max * D * (L.T_max + 1) * 10));
   chk(alloc(&pl->dbg_d, (size_t)L.E_max * D * L.T_max));
@@ -879,6 +885,15 @@ int create_planner(const aero_limits_t* limits, aero_planner_t** out, bool batch
   if (e == cudaSuccess) e = split_attributes();
   if (e == cudaSuccess) e = cudaMemset(pl->counter, 0, kCounterWords * sizeof(unsigned int));
   if (e == cudaSuccess) e = cudaMemset(pl->status, 0, sizeof(int));
+  if (e == cudaSuccess && pl->warm_grid) {
+    WarmGrid wg{};
+    for (int i = 0; i < kWarmList; ++i) {
+      std::memcpy(&wg.pts[i].w, &i, sizeof(i));  // the point's item
+      wg.cand[i] = (uint32_t)i;
+    }
+    wg.range = make_int2(0, kWarmList);
+    e = cudaMemcpy(pl->warm_grid, &wg, sizeof(wg), cudaMemcpyHostToDevice);
+  }
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) {
     cudaGetLastError();

@@ -132,6 +132,17 @@ struct GridView {
   float origin, inv_h;
 };
 
+// A grid of one cell that every position up to 10^6 m from the start falls into, with a
+// list long enough for every part of the scans: what a warm-up run queries while the
+// planner's own grid may still be written.  Written once, when the planner is created.
+constexpr int kWarmList = 16;
+constexpr float kWarmOrigin = -1e6f, kWarmInvH = 5e-7f;
+struct WarmGrid {
+  float4 pts[kWarmList];
+  uint32_t cand[kWarmList];
+  int2 range;
+};
+
 struct CostParams {
   float Q_track, Q_vnorm, Q_c, Q_cd, Q_p, Q_v, Q_q;
   float C_col, a_col, d_min, d_max;
@@ -192,6 +203,7 @@ struct UpdateArgs {
   int* status;             // bit 0: a normaliser eta was not a positive finite number
   float* warm;             // scratch of the warm-up runs of the update's code: E regions of
                            // warm_words(E, T) floats; null: no warm-up runs
+  const WarmGrid* warm_grid;  // the update launch's warm-up runs query this grid
   unsigned int* done;      // the update launch: {finished CTAs of the one-lane pass, exit
                            // ticket}, both reset by its last CTA; or null
 };

@@ -851,8 +851,14 @@ __global__ void __launch_bounds__(NT, 6) k_rollout(RolloutArgs a) {
 // runs too.  The update runs once per launch, so without it its instructions
 // would be fetched cold (from DRAM once the L2 has been overwritten) on the
 // critical path; the warm-up run's results are discarded.  It may read
-// partials that other CTAs are writing: every access of the update stays in
-// bounds whatever the values read.  Every thread of the CTA calls it.
+// partials and nominals that other CTAs are writing (through L2): every access of the
+// update stays in bounds whatever the values read.
+// grid: null, or the grid to query and the region's nominals as the guides, for a run
+// that may overlap the launches that write the planner's grid and guides.  Lists and
+// ranges are read through the non-coherent path, which is for data that nothing writes
+// meanwhile: what it read early could still be in this SM's L1 when the real run reads
+// the same lists, in another order and with other ranges once they are pruned.
+// Every thread of the CTA calls it.
 //
 // The region holds the Stage II states of instance e alone, where the update writes
 // those of instance e at e (T + 1) 10 from a.stage2_x: from where that pointer starts
@@ -877,7 +883,7 @@ constexpr bool warm_regions_hold() {
 }
 static_assert(warm_regions_hold(), "every warm-up run stays in its region");
 
-__device__ __forceinline__ void warm_setup(UpdateArgs* s_ua, const UpdateArgs& ua, int e) {
+__device__ __forceinline__ void warm_setup(UpdateArgs* s_ua, const UpdateArgs& ua, int e, const WarmGrid* grid) {
   const int E = ua.E, T = ua.T;
   float* const sc = ua.warm + (size_t)e * warm_words(E, T);
   if (threadIdx.x == 0) {
@@ -889,9 +895,14 @@ __device__ __forceinline__ void warm_setup(UpdateArgs* s_ua, const UpdateArgs& u
     s_ua->counter = reinterpret_cast<unsigned int*>(s_ua->best_idx + 1);
     s_ua->status = reinterpret_cast<int*>(s_ua->counter + 1);
     s_ua->dbg_pre = nullptr;
+    if (grid != nullptr) {
+      s_ua->grid = GridView{&grid->range, grid->cand, grid->pts, 1, kWarmOrigin, kWarmInvH};
+      s_ua->guides = sc;
+    }
     *s_ua->counter = (unsigned)(E - 1);
   }
-  for (int i = threadIdx.x; i < 4 * T; i += blockDim.x) sc[(size_t)e * T * 4 + i] = ua.u_nom[(size_t)e * T * 4 + i];
+  for (int i = threadIdx.x; i < 4 * T; i += blockDim.x)
+    sc[(size_t)e * T * 4 + i] = __ldcg(ua.u_nom + (size_t)e * T * 4 + i);
   __syncthreads();
 }
 
@@ -925,7 +936,7 @@ __global__ void __launch_bounds__(ST, 2) k_rollout_split(RolloutArgs a, UpdateAr
   if (warm) pdl_wait();  // the warm-up run reads the grid
   block_copy_param(&s_ua, &ua);
   __syncthreads();
-  if (warm) warm_setup(&s_ua, ua, 0);
+  if (warm) warm_setup(&s_ua, ua, 0, nullptr);
   extern __shared__ __align__(16) unsigned char fused_smem[];  // the split pass's, free again
   update_unit<ST>(s_ua, e, s_ua.final_stage != 0, fused_smem);
 }
@@ -941,7 +952,10 @@ __global__ void __launch_bounds__(ST, 2) k_rollout_split(RolloutArgs a, UpdateAr
 // instance's update as a warm-up run (warm_setup) before it waits for Stage I:
 // the launch is programmatic, so its CTAs start as soon as the last CTAs of
 // Stage I have started, and the warm-up runs overlap Stage I's last wave; the
-// real update then finds its code in L2 and this SM's instruction caches.  A
+// real update then finds its code in L2 and this SM's instruction caches.  Stage I's
+// CTAs count as started before they have waited for their own predecessor: where all
+// of them fit at once, the warm-up runs overlap the grid's launches too, so they
+// query a grid of their own (a.warm_grid).  A
 // CTA that starts after Stage I has finished (every one of its CTAs counted
 // in a.done[0]: the launch was not overlapped) skips the warm-up run.  One
 // call site for both runs (the same code).
@@ -959,7 +973,7 @@ __global__ void __launch_bounds__(ST) k_update(UpdateArgs a) {
     else pdl_trigger();
     block_copy_param(&s_a, &a);
     __syncthreads();
-    if (run == 0) warm_setup(&s_a, a, blockIdx.x);
+    if (run == 0) warm_setup(&s_a, a, blockIdx.x, a.warm_grid);
     update_unit<ST>(s_a, blockIdx.x, s_a.final_stage != 0, upd_smem);
     __syncthreads();  // s_a and the scratch free for the next run
   }
