@@ -370,7 +370,7 @@ __device__ float warp_cost_grad(const float4* __restrict__ U, float4* __restrict
     const int j = 32 * r + lane;
     const bool on = j < T;
     const float4 u = on ? su[j] : make_float4(0.f, 0.f, 0.f, 0.f);
-    float4 m = on ? rk4_attitude_coefs(u, dp) : make_float4(1.f, 0.f, 0.f, 0.f);
+    float4 m = on ? attitude_factor(u, dp) : make_float4(1.f, 0.f, 0.f, 0.f);
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
       const float4 y = shfl_up4(m, o);
