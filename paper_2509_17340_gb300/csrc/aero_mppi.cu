@@ -269,15 +269,16 @@ GridGeom make_grid(const aero_params_t& p, int64_t n_items, int64_t cap, int gma
   g.reach = p.d_max * (1.0f + 1e-3f) + 1e-4f;
   float h = !coarse && (int64_t)kFineDup * n_items <= cap ? 0.5f * p.d_max : p.d_max * 1.0625f;
   float E = p.r_max + g.reach + h;
-  int G = (int)std::ceil(2.0f * E / h);
-  if (G > gmax) {
+  // compared as floats: far more cells than an int counts is a conversion without a
+  // defined result (negative on x86, which would pass for few cells)
+  float cells = std::ceil(2.0f * E / h);
+  if (!(cells <= (float)gmax)) {
     // coarser cells: E grows with h, so solve h = 2 (r_max + reach + h) / gmax
     h = 2.0f * (p.r_max + g.reach) / ((float)gmax - 2.5f);
     E = p.r_max + g.reach + h;
-    G = (int)std::ceil(2.0f * E / h);
-    if (G > gmax) G = gmax;
+    cells = std::ceil(2.0f * E / h);
   }
-  g.G = G;
+  g.G = cells <= (float)gmax ? (int)cells : gmax;
   g.h = h;
   g.inv_h = 1.0f / h;
   g.origin = -E;
