@@ -3,6 +3,7 @@
 // the launch sequence of one step.  Host code is compiled with
 // -ffp-contract=off so that R(q0), the goal offset and the edge tables follow
 // the stated binary32/binary64 operation order exactly.
+#include <cfloat>
 #include <cmath>
 #include <cstdint>
 #include <cstdio>
@@ -456,7 +457,8 @@ void make_step_args(aero_planner* pl, const aero_state_t* x0, const float* cloud
   pa.n = n;
   for (int i = 0; i < 3; ++i) pa.p0[i] = x0->p[i];
   for (int i = 0; i < 9; ++i) pa.R[i] = R[i];
-  pa.rmax2 = rmax2;
+  pa.rmax2 = std::fmin(rmax2, FLT_MAX);
+  pa.unbounded = std::isinf(rmax2);
   pa.A = p.fine_az;
   pa.El = p.fine_el;
   pa.check_lo = a.check_lo;
@@ -468,6 +470,8 @@ void make_step_args(aero_planner* pl, const aero_state_t* x0, const float* cloud
   // 1e-5 rad, and what the multiplication into units of cones rounds off
   pa.az_eps = 1e-5f * pa.az_scale + 1e-6f * (float)p.fine_az;
   pa.el_eps = 1e-5f * pa.el_inv + 1e-6f * ((float)p.fine_el + std::fabs(p.el_lo) * pa.el_inv);
+  // the guesses' quotients end at coordinates of 2^126: beyond, the predicates decide
+  if (pa.unbounded) pa.az_eps = pa.el_eps = 1.0f;
   pa.keys = pl->keys;
   pa.item_flag = a.raw ? pl->item_flag : nullptr;
   pa.counts = pl->part_counts;

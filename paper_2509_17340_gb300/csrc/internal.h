@@ -56,7 +56,8 @@ struct PartitionArgs {
   int64_t n;
   float p0[3];
   float R[9];      // R(q0) in binary32, row-major
-  float rmax2;     // r_max * r_max in binary32
+  float rmax2;     // r_max * r_max in binary32, at most the largest finite number
+  int unbounded;   // r_max * r_max is infinite: finite points of infinite r^2 are inside
   int A, El;
   int check_lo, check_hi;
   int filter;      // read a cone's key before its atomic minimum (dense clouds)

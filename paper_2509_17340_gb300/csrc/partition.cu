@@ -150,9 +150,12 @@ __device__ __forceinline__ int cone_of(const PartitionArgs& a, const SmemTables&
   to_body(a.R, dx, dy, dz, b);
   const float rxy2 = add(mul(b[0], b[0]), mul(b[1], b[1]));
   const float r2 = add(rxy2, mul(b[2], b[2]));
-  // a non-finite coordinate makes every component of b infinite or NaN
-  if (!(r2 > 0.0f && r2 <= a.rmax2))
-    return isfinite(pt.x) && isfinite(pt.y) && isfinite(pt.z) ? kOutside : kNonFinite;
+  // a non-finite coordinate makes every component of b infinite or NaN, and r2 above the
+  // (finite) bound
+  if (!(r2 > 0.0f && r2 <= a.rmax2)) {
+    if (!(isfinite(pt.x) && isfinite(pt.y) && isfinite(pt.z))) return kNonFinite;
+    if (!(a.unbounded && r2 == INFINITY)) return kOutside;
+  }
   const float ga = (atan2_guess(b[1], b[0]) + 3.141592654f) * a.az_scale;
   const float ge = (atan2_guess(b[2], fast_sqrt(rxy2)) - a.el_lo) * a.el_inv;
   int ia = __float2int_rd(ga), je = __float2int_rd(ge);
