@@ -472,6 +472,9 @@ void make_step_args(aero_planner* pl, const aero_state_t* x0, const float* cloud
   pa.el_eps = 1e-5f * pa.el_inv + 1e-6f * ((float)p.fine_el + std::fabs(p.el_lo) * pa.el_inv);
   // the guesses' quotients end at coordinates of 2^126: beyond, the predicates decide
   if (pa.unbounded) pa.az_eps = pa.el_eps = 1.0f;
+  // cones wider than half a turn (a span of more than a whole one): an edge's predicate,
+  // the sine of the angle past it, changes its sign within the cone, so it decides
+  if (pa.el_inv < 1.0f / 3.0f) pa.el_eps = 1.0f;
   pa.keys = pl->keys;
   pa.item_flag = a.raw ? pl->item_flag : nullptr;
   pa.counts = pl->part_counts;

@@ -1,6 +1,7 @@
 """The partition at the ends of what its parameters accept: a range bound whose square is
 infinite in binary32, where finite points beyond 1.8e19 m are inside and non-finite ones
-are still left out."""
+are still left out; elevation spans of more than a turn, whose cones are wider than half
+a turn."""
 import numpy as np
 import pytest
 
@@ -42,4 +43,19 @@ def test_range_bound_beyond_binary32(aero, orc, r_max, A, El, turned):  # noqa: 
     keys, kept = orc.partition(w.cloud, w.p0, w.q0, P)
     g = _step(aero, w, P)
     assert list(g["point_counts"]) == [n, 300, kept]
+    assert np.array_equal(g["keys"], keys)
+
+
+@pytest.mark.parametrize("El,lo,hi", [(2, -6.0, 2.0), (2, -2.0, 6.0), (3, -5.0, 5.0), (1, -10.0, 10.0), (3, -4.0, 4.0)])
+def test_cones_wider_than_half_a_turn(aero, orc, El, lo, hi):  # noqa: F811
+    w = I.make_workload("plain", seed=El)
+    rng = np.random.default_rng([El, int(10 * hi)])
+    w.p0 = np.zeros(3, np.float32)
+    d = rng.normal(size=(6000, 3))
+    w.cloud = (d / np.linalg.norm(d, axis=1, keepdims=True) * rng.uniform(0.1, 9.0, (6000, 1))).astype(np.float32)
+    P = w.params
+    P.update(E=1, M_h=1, M_v=1, K=32, T=4, fine_az=120, fine_el=El, pool_az=1, pool_el=1, el_lo=lo, el_hi=hi)
+    keys, kept = orc.partition(w.cloud, w.p0, w.q0, P)
+    g = _step(aero, w, P)
+    assert list(g["point_counts"]) == [6000, 0, kept]
     assert np.array_equal(g["keys"], keys)
