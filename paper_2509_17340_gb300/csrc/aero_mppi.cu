@@ -749,7 +749,7 @@ int enqueue_step(aero_planner* pl, const aero_state_t* x0, const float* cloud, i
     a.ua.final_stage = it == p.iters - 1;
     ranges.next("aero stage I");
     mark(AERO_STAGE_ROLLOUT, 4 + 4 * it);
-    if ((e = launch_rollout(a.ra, a.ua, s)) != cudaSuccess) return cuda_fail(e);
+    if ((e = launch_rollout(a.ra, a.ua, it > 0 || !prune, s)) != cudaSuccess) return cuda_fail(e);
     mark(AERO_STAGE_ROLLOUT, 5 + 4 * it);
     ranges.next("aero update");
     mark(AERO_STAGE_UPDATE, 6 + 4 * it);
@@ -1551,18 +1551,19 @@ cudaError_t batch_graph(aero_batch* b, int n, int max_iters, int has1, int has4,
   if (le == cudaSuccess) le = launch_batch_scatter(v, S * b->occ_grid[3], c);
   if (le == cudaSuccess && prune) le = launch_batch_prune(v, S * b->occ_grid[4], c);
   for (int it = 0; it < max_iters && le == cudaSuccess; ++it) {
+    const bool overlap = it > 0 || !prune;
     if (has1 && has4) {
       le = cudaEventRecord(b->fork, c);
       if (le == cudaSuccess) le = cudaStreamWaitEvent(b->cap2, b->fork, 0);
       if (le == cudaSuccess)
-        le = launch_batch_rollout(v, 4, it, roll_blocks(1), cfg.dynamic_queue, 0, spc, b->cap2);
+        le = launch_batch_rollout(v, 4, it, roll_blocks(1), cfg.dynamic_queue, 0, spc, true, b->cap2);
       if (le == cudaSuccess)
-        le = launch_batch_rollout(v, 1, it, roll_blocks(0), cfg.dynamic_queue, six, spc, c);
+        le = launch_batch_rollout(v, 1, it, roll_blocks(0), cfg.dynamic_queue, six, spc, overlap, c);
       if (le == cudaSuccess) le = cudaEventRecord(b->join, b->cap2);
       if (le == cudaSuccess) le = cudaStreamWaitEvent(c, b->join, 0);
     } else {
       le = launch_batch_rollout(v, has4 ? 4 : 1, it, roll_blocks(has4 ? 1 : 0), cfg.dynamic_queue,
-                                has4 ? 0 : six, spc, c);
+                                has4 ? 0 : six, spc, overlap, c);
     }
     if (le == cudaSuccess) le = launch_batch_update(v, it, S * b->occ_roll[2], c);
   }

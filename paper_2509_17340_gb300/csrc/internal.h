@@ -284,9 +284,10 @@ cudaError_t launch_batch_prune(const BatchView& v, int blocks, cudaStream_t s);
 // lanes 1 or 4; dynamic: take units from the work queue, else stride by the grid;
 // six: the one-lane kernel compiled for six resident CTAs per SM (fewer
 // registers) instead of five; samples_per_cta: the one-lane pass's CTA size
-// (64, 128 or 256; the items' partial rows were laid out for it)
+// (64, 128 or 256; the items' partial rows were laid out for it); overlap: as
+// launch_rollout's
 cudaError_t launch_batch_rollout(const BatchView& v, int lanes, int it, int blocks, int dynamic,
-                                 int six, int samples_per_cta, cudaStream_t s);
+                                 int six, int samples_per_cta, bool overlap, cudaStream_t s);
 cudaError_t launch_batch_update(const BatchView& v, int it, int blocks, cudaStream_t s);
 
 // Resident CTAs per SM: {partition, count, scan, scatter, prune} and {rollout with one
@@ -325,8 +326,9 @@ struct CostGradArgs {
 };
 
 // Stage I; the split pass (lanes_per_sample 4) also runs the update `ua` in
-// the last CTA of every instance, the others leave it to launch_update.
-cudaError_t launch_rollout(const RolloutArgs& a, const UpdateArgs& ua, cudaStream_t s);
+// the last CTA of every instance, the others leave it to launch_update.  overlap: the
+// one-lane pass may start while the launch in front of it still runs.
+cudaError_t launch_rollout(const RolloutArgs& a, const UpdateArgs& ua, bool overlap, cudaStream_t s);
 bool rollout_runs_update(const RolloutArgs& a);
 // Sets the kernels' shared-memory limits (once per device).
 cudaError_t split_attributes();

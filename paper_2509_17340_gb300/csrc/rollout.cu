@@ -1182,16 +1182,16 @@ cudaError_t batch_rollout_occupancy(int out[6], int T_max) {
 }
 
 cudaError_t launch_batch_rollout(const BatchView& v, int lanes, int it, int blocks, int dynamic,
-                                 int six, int samples_per_cta, cudaStream_t s) {
+                                 int six, int samples_per_cta, bool overlap, cudaStream_t s) {
   if (lanes == 4)
     return launch_ks(k_b_rollout<4, 2>, dim3(blocks), dim3(ST), split_smem_bytes(v.T_max), s, true, v,
                      it, dynamic);
   if (samples_per_cta == 64)
-    return launch_k(k_b_rollout<1, 12, 64>, dim3(blocks), dim3(64), s, true, v, it, dynamic);
+    return launch_k(k_b_rollout<1, 12, 64>, dim3(blocks), dim3(64), s, overlap, v, it, dynamic);
   if (samples_per_cta == 256)
-    return launch_k(k_b_rollout<1, 3, 256>, dim3(blocks), dim3(256), s, true, v, it, dynamic);
-  if (six) return launch_k(k_b_rollout<1, 6>, dim3(blocks), dim3(NT), s, true, v, it, dynamic);
-  return launch_k(k_b_rollout<1, 5>, dim3(blocks), dim3(NT), s, true, v, it, dynamic);
+    return launch_k(k_b_rollout<1, 3, 256>, dim3(blocks), dim3(256), s, overlap, v, it, dynamic);
+  if (six) return launch_k(k_b_rollout<1, 6>, dim3(blocks), dim3(NT), s, overlap, v, it, dynamic);
+  return launch_k(k_b_rollout<1, 5>, dim3(blocks), dim3(NT), s, overlap, v, it, dynamic);
 }
 
 cudaError_t launch_batch_update(const BatchView& v, int it, int blocks, cudaStream_t s) {
@@ -1201,7 +1201,15 @@ cudaError_t launch_batch_update(const BatchView& v, int it, int blocks, cudaStre
 
 bool rollout_runs_update(const RolloutArgs& a) { return a.lanes_per_sample == 4; }
 
-cudaError_t launch_rollout(const RolloutArgs& a, const UpdateArgs& ua, cudaStream_t s) {
+// The one-lane pass after the list pruning (overlap false) is an ordinary launch.  Its
+// lists live on L1 hits, and an SM keeps its split between L1 and shared memory while
+// it is never empty: a launch that starts under the pruning's last blocks (45 KB of
+// shared memory each) runs with the little L1 that these left.  Large clutter (E = 32,
+// K = 8192, T = 64), a whole step: 375 us overlapped, 351 in order, 349 unpruned; two
+// denser scenes 398 -> 360 and 412 -> 373; 32 planners of 3.2 M sample-steps 2250 ->
+// 2177, 64 of 0.5 M 1288 -> 1244.  The split pass sets its own split, and the
+// two launch forms measure alike (within 4 us, the overlapped one ahead).
+cudaError_t launch_rollout(const RolloutArgs& a, const UpdateArgs& ua, bool overlap, cudaStream_t s) {
   if (a.lanes_per_sample == 4) {
     cudaError_t e = split_attributes();
     // the carveout is a hint: a launch being captured into a graph keeps the
@@ -1213,8 +1221,8 @@ cudaError_t launch_rollout(const RolloutArgs& a, const UpdateArgs& ua, cudaStrea
     const dim3 grid((unsigned)a.nb * a.E + (ua.warm != nullptr ? 1u : 0u));
     return launch_ks(k_rollout_split, grid, dim3(ST), split_smem_bytes(a.T), s, true, a, ua);
   }
-  if (a.list_thr > 0) return launch_k(k_rollout<true>, dim3(a.nb, a.E), dim3(NT), s, true, a);
-  return launch_k(k_rollout<false>, dim3(a.nb, a.E), dim3(NT), s, true, a);
+  if (a.list_thr > 0) return launch_k(k_rollout<true>, dim3(a.nb, a.E), dim3(NT), s, overlap, a);
+  return launch_k(k_rollout<false>, dim3(a.nb, a.E), dim3(NT), s, overlap, a);
 }
 
 cudaError_t launch_update(const UpdateArgs& a, cudaStream_t s) {
