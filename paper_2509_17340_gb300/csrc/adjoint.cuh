@@ -625,7 +625,8 @@ __device__ __forceinline__ RefineScratch refine_layout(unsigned char* base, int 
 
 // `steps` clamped gradient steps u <- clamp(u - alpha dS/du) on the nominal u
 // (shared, T <= kThreads entries), by all kThreads threads of the CTA.
-template <int kThreads>
+// kEither: the grid's entries may be the points themselves (grid_point).
+template <int kThreads, bool kEither>
 __device__ void block_refine(float4* u, const float* guide, int T, const float* x0,
                              const DynParams& dp, const CostParams& cp, const GridView& grid,
                              const float* umin, const float* umax, int steps, float alpha,
@@ -668,7 +669,7 @@ __device__ void block_refine(float4* u, const float* guide, int T, const float* 
       float best = dmax2;
       int bitem = -1;
       for (int c = 0; c < n; ++c) {
-        const float4 p = grid_point(grid, q.x + first + c);
+        const float4 p = grid_point<kEither>(grid, q.x + first + c);
         const float d2 = dist2_to(p, x1[0], x1[1], x1[2]);
         const int item = point_item(p);
         if (d2 < best || (d2 == best && bitem >= 0 && item < bitem)) {

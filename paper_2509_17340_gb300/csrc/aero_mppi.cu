@@ -134,8 +134,9 @@ struct aero_planner {
   int* grid_local = nullptr;  // G^3 + 1 tile-local exclusive prefix
   int* tile_sum = nullptr;
   int* tile_off = nullptr;
-  uint32_t* cand = nullptr;   // candidate entries: item indices
+  uint32_t* cand = nullptr;   // candidate entries: item indices; a batch slot has room for points
   float4* cand_pts = nullptr; // collision point of every item, minus p0
+  bool last_own = false;      // the last step's entries were the points themselves
   int2* grid_range = nullptr; // G^3 {first entry, count}
   int cand_cap = 0;
   int grid_max = kGridMax;    // cells per axis the grid arrays can hold
@@ -425,7 +426,7 @@ int lanes_of(const aero_params_t& p, int64_t quad_max) {
 
 void make_step_args(aero_planner* pl, const aero_state_t* x0, const float* cloud, int64_t n,
                     const float* goal, const aero_params_t& p, float* u_nom, float* u_best,
-                    float* cand, int32_t* best_idx, int lanes, bool coarse, StepArgs& a,
+                    float* cand, int32_t* best_idx, int lanes, bool coarse, bool own, StepArgs& a,
                     int samples_per_cta = kRolloutThreads) {
   a.ncell = p.fine_az * p.fine_el;
   // the edge tables depend only on the partition geometry: recomputed when it changes
@@ -492,6 +493,7 @@ void make_step_args(aero_planner* pl, const aero_state_t* x0, const float* cloud
   ca.local = pl->grid_local;
   ca.tile_off = pl->tile_off;
   ca.cand = pl->cand;
+  ca.own = own ? reinterpret_cast<float4*>(pl->cand) : nullptr;
   ca.pts = pl->cand_pts;
   ca.status = pl->status;
   ca.reset_keys = nullptr;
@@ -538,7 +540,7 @@ void make_step_args(aero_planner* pl, const aero_state_t* x0, const float* cloud
   for (int i = 0; i < 3; ++i) cp.v_goal[i] = p.v_goal[i];
   for (int i = 0; i < 4; ++i) cp.q_goal[i] = p.q_goal[i];
   DynParams dp{p.dt, 1.0f / p.mass, p.g};
-  GridView gv{pl->grid_range, pl->cand, pl->cand_pts, a.grid.G, a.grid.origin, a.grid.inv_h};
+  GridView gv{pl->grid_range, pl->cand, pl->cand_pts, a.grid.G, a.grid.origin, a.grid.inv_h, ca.own};
   const float x0v[10] = {0.0f, 0.0f, 0.0f, x0->q[0], x0->q[1], x0->q[2], x0->q[3],
                          x0->v[0], x0->v[1], x0->v[2]};
   a.lanes = lanes;
@@ -633,6 +635,7 @@ void note_step(aero_planner* pl, const aero_params_t& p, const StepArgs& a) {
   pl->have_step = true;
   pl->last = p;
   pl->last_grid = a.grid;
+  pl->last_own = false;
   pl->last_ntiles = a.ntiles;
   pl->last_nb = a.nb;
   pl->last_part_slots = partition_blocks(a.pa.n);
@@ -667,7 +670,7 @@ int enqueue_step(aero_planner* pl, const aero_state_t* x0, const float* cloud, i
                  float* cand, int32_t* best_idx, cudaStream_t s, const float* mapped = nullptr) {
   StepArgs a;
   make_step_args(pl, x0, cloud, n, goal, p, u_nom, u_best, cand, best_idx,
-                 lanes_of(p, kQuadMaxSamples), false, a);
+                 lanes_of(p, kQuadMaxSamples), false, false, a);
   if (mapped) {
     a.pa.cloud = mapped;
     a.pa.copy_to = const_cast<float*>(cloud);
@@ -826,7 +829,7 @@ int aero_create(const aero_limits_t* limits, aero_planner_t** out) {
 namespace {
 
 // batch_slot: the workspace of a batch's item slot, whose candidate entries
-// hold the points (16 bytes); a single planner's entries are 4-byte item
+// may be the points (16 bytes); a single planner's entries are 4-byte item
 // indices, so the same bytes hold four times the entries and the every-point
 // set gets room for the finer cells (216 entries per kept point).
 int create_planner(const aero_limits_t* limits, aero_planner_t** out, bool batch_slot) {
@@ -866,7 +869,7 @@ int create_planner(const aero_limits_t* limits, aero_planner_t** out, bool batch
   chk(alloc(&pl->grid_local, kGridCellsMax + 1));
   chk(alloc(&pl->tile_sum, kMaxTiles));
   chk(alloc(&pl->tile_off, kMaxTiles + 1));
-  chk(alloc(&pl->cand, cap));
+  chk(dev_malloc((void**)&pl->cand, (batch_slot ? sizeof(float4) : sizeof(uint32_t)) * (size_t)(cap > 0 ? cap : 1)));
   chk(alloc(&pl->cand_pts, std::max<int64_t>(L.fine_cells_max, pl->raw_max)));
   chk(alloc(&pl->grid_range, kGridCellsMax));
   chk(alloc(&pl->partials, (size_t)L.E_max * nbmax * (4 + 4 * L.T_max)));
@@ -1065,6 +1068,7 @@ int aero_get_debug(aero_planner_t* pl, int32_t what, void* dst, size_t bytes, vo
       const size_t ne = (size_t)(n_entries < g.cap ? n_entries : g.cap);
       const size_t need = sizeof(float4) * ne;
       if (bytes < need) return AERO_ERR_INVALID_ARG;
+      if (pl->last_own) return cuda_fail(cudaMemcpy(dst, pl->cand, need, cudaMemcpyDefault));
       const size_t n_items = (size_t)std::max<int64_t>(pl->lim.fine_cells_max, pl->raw_max);
       std::vector<uint32_t> idx(ne);
       std::vector<float4> pts(n_items), out(ne);
@@ -1548,7 +1552,7 @@ cudaError_t batch_graph(aero_batch* b, int n, int max_iters, int has1, int has4,
   cudaError_t le = launch_batch_partition(v, S * b->occ_grid[0], c);
   if (le == cudaSuccess) le = launch_batch_count(v, S * b->occ_grid[1], c);
   if (le == cudaSuccess) le = launch_batch_scan(v, S * b->occ_grid[2], c);
-  if (le == cudaSuccess) le = launch_batch_scatter(v, S * b->occ_grid[3], c);
+  if (le == cudaSuccess) le = launch_batch_scatter(v, S * b->occ_grid[3], !prune, c);
   if (le == cudaSuccess && prune) le = launch_batch_prune(v, S * b->occ_grid[4], c);
   for (int it = 0; it < max_iters && le == cudaSuccess; ++it) {
     const bool overlap = it > 0 || !prune;
@@ -1556,14 +1560,14 @@ cudaError_t batch_graph(aero_batch* b, int n, int max_iters, int has1, int has4,
       le = cudaEventRecord(b->fork, c);
       if (le == cudaSuccess) le = cudaStreamWaitEvent(b->cap2, b->fork, 0);
       if (le == cudaSuccess)
-        le = launch_batch_rollout(v, 4, it, roll_blocks(1), cfg.dynamic_queue, 0, spc, true, b->cap2);
+        le = launch_batch_rollout(v, 4, it, roll_blocks(1), cfg.dynamic_queue, 0, spc, !prune, true, b->cap2);
       if (le == cudaSuccess)
-        le = launch_batch_rollout(v, 1, it, roll_blocks(0), cfg.dynamic_queue, six, spc, overlap, c);
+        le = launch_batch_rollout(v, 1, it, roll_blocks(0), cfg.dynamic_queue, six, spc, !prune, overlap, c);
       if (le == cudaSuccess) le = cudaEventRecord(b->join, b->cap2);
       if (le == cudaSuccess) le = cudaStreamWaitEvent(c, b->join, 0);
     } else {
       le = launch_batch_rollout(v, has4 ? 4 : 1, it, roll_blocks(has4 ? 1 : 0), cfg.dynamic_queue,
-                                has4 ? 0 : six, spc, overlap, c);
+                                has4 ? 0 : six, spc, !prune, overlap, c);
     }
     if (le == cudaSuccess) le = launch_batch_update(v, it, S * b->occ_roll[2], c);
   }
@@ -1607,7 +1611,18 @@ int batch_enqueue(aero_batch* b, const aero_batch_item_t* items, int n, cudaStre
   std::vector<int> lanes(n), T(n);
   std::vector<int> tab_changed;
   int max_iters = 0, has1 = 0, has4 = 0;
-  int64_t steps = 0;  // sample-steps of all items: lists are pruned from kPruneBatchSteps per item on
+  // Lists are pruned from kPruneBatchSteps sample-steps per item on, unless an item's
+  // collision set is every kept point: the coarse cells' lists of those cost more to
+  // prune than Stage I saves (8 planners of 2.6 M sample-steps and up to 60,000 points:
+  // 13.1 ms pruned, 10.9 with the entries' own points).
+  int64_t steps = 0;
+  bool raw = false;
+  for (int i = 0; i < n; ++i) {
+    const aero_params_t& p = items[i].params;
+    steps += (int64_t)p.E * p.K * p.T * p.iters;
+    raw = raw || p.collision_set == 1;
+  }
+  const bool prune = steps >= kPruneBatchSteps * n && !raw;
   for (int k = 0; k < kPreCount; ++k) pre[k * (n + 1)] = 0;
   for (int i = 0; i < n; ++i) {
     const aero_batch_item_t& it = items[i];
@@ -1626,7 +1641,7 @@ int batch_enqueue(aero_batch* b, const aero_batch_item_t* items, int n, cudaStre
     }
     StepArgs a;
     make_step_args(pl, &it.x0, it.cloud_xyz, it.n_points, it.goal, p, u_nom, u_best, cand, best,
-                   lanes_of(p, cfg.quad_max_samples), cfg.coarse_cells != 0, a, spc_of(cfg));
+                   lanes_of(p, cfg.quad_max_samples), cfg.coarse_cells != 0, !prune, a, spc_of(cfg));
     BatchItem& bi = hi[i];
     bi.pa = a.pa;
     bi.ca = a.ca;
@@ -1668,7 +1683,6 @@ int batch_enqueue(aero_batch* b, const aero_batch_item_t* items, int n, cudaStre
     meta[i] = {a.grid, a.ntiles, a.nb};
     lanes[i] = a.lanes;
     T[i] = p.T;
-    steps += (int64_t)p.E * p.K * p.T * p.iters;
     if (p.iters > max_iters) max_iters = p.iters;
     (a.lanes == 4 ? has4 : has1) = 1;
   }
@@ -1691,7 +1705,7 @@ int batch_enqueue(aero_batch* b, const aero_batch_item_t* items, int n, cudaStre
   }
 
   cudaGraphExec_t exec = nullptr;
-  if ((e = batch_graph(b, n, max_iters, has1, has4, steps >= kPruneBatchSteps * n, cfg, &exec)) != cudaSuccess) return cuda_fail(e);
+  if ((e = batch_graph(b, n, max_iters, has1, has4, prune, cfg, &exec)) != cudaSuccess) return cuda_fail(e);
   // workspaces whose counts or keys may be stale (new slot, interrupted step)
   for (int i = 0; i < n; ++i) {
     aero_planner* pl = b->planners[i];
@@ -1721,6 +1735,7 @@ int batch_enqueue(aero_batch* b, const aero_batch_item_t* items, int n, cudaStre
     pl->have_step = true;
     pl->last = items[i].params;
     pl->last_grid = meta[i].grid;
+    pl->last_own = !prune;
     pl->last_ntiles = meta[i].ntiles;
     pl->last_part_slots = (int)((items[i].n_points + kPartChunk - 1) / kPartChunk);
     pl->last_n_points = items[i].n_points;

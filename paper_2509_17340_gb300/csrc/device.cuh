@@ -416,9 +416,22 @@ __device__ __forceinline__ float dist2_to(const float4 q, float px, float py, fl
 
 // The collision point of candidate entry e of the grid; its w holds the bits of
 // the point's item index (the position of the point in the collision set: the fine
-// cone of a P_f point, the index of a kept point).
+// cone of a P_f point, the index of a kept point).  kEither: the entries may be the
+// points themselves (batched steps), found by g.own.
+template <bool kEither = false>
 __device__ __forceinline__ float4 grid_point(const GridView& g, int e) {
+  if (kEither && g.own != nullptr) return __ldg(g.own + e);
   return __ldg(g.pts + __ldg(g.cand + e));
+}
+
+// The same where the form is known at compile time, for the per-entry loop of the
+// one-lane pass.
+template <bool kOwn>
+__device__ __forceinline__ float4 grid_point_of(const GridView& g, int e) {
+  if constexpr (kOwn)
+    return __ldg(g.own + e);
+  else
+    return __ldg(g.pts + __ldg(g.cand + e));
 }
 
 __device__ __forceinline__ int point_item(float4 p) { return __float_as_int(p.w); }
@@ -463,19 +476,27 @@ __device__ __forceinline__ float warp_split_min(const GridView& g, int2 range, f
 // min(best, squared distances to the points of the n candidate entries from
 // `first`), kW entries per round so that kW loads are in flight; the last
 // round repeats its first entry in place of the missing ones (the minimum is
-// exact in any order).
-template <int kW = 4>
+// exact in any order).  kEither: as grid_point's.
+template <int kW = 4, bool kEither = false>
 __device__ __forceinline__ float scan_min(const GridView& g, int first, int n, float px, float py,
                                           float pz, float best) {
-  const uint32_t* E = g.cand + first;
+  const bool own = kEither && g.own != nullptr;
+  const uint32_t* E = own ? nullptr : g.cand + first;
+  const float4* P = own ? g.own + first : g.pts;
   for (int t = 0; t < n; t += kW) {
     float4 c[kW];
-    uint32_t id[kW];
-    id[0] = __ldg(E + t);
+    if (own) {
+      c[0] = __ldg(P + t);
 #pragma unroll
-    for (int i = 1; i < kW; ++i) id[i] = t + i < n ? __ldg(E + t + i) : id[0];
+      for (int i = 1; i < kW; ++i) c[i] = t + i < n ? __ldg(P + t + i) : c[0];
+    } else {
+      uint32_t id[kW];
+      id[0] = __ldg(E + t);
 #pragma unroll
-    for (int i = 0; i < kW; ++i) c[i] = __ldg(g.pts + id[i]);
+      for (int i = 1; i < kW; ++i) id[i] = t + i < n ? __ldg(E + t + i) : id[0];
+#pragma unroll
+      for (int i = 0; i < kW; ++i) c[i] = __ldg(P + id[i]);
+    }
     float m = dist2_to(c[0], px, py, pz);
 #pragma unroll
     for (int i = 1; i < kW; ++i) m = fminf(m, dist2_to(c[i], px, py, pz));

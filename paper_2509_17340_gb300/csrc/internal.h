@@ -84,7 +84,9 @@ struct CandArgs {
   int* fill;           // G^3 + 1: fill cursors of the scatter pass; zeroed by the scan
   const int* local;    // tile-local exclusive prefix of the counts (scatter pass)
   const int* tile_off; // exclusive prefix of the tile totals (scatter pass)
-  uint32_t* cand;      // candidate entries (scatter pass): item indices into pts
+  // candidate entries (scatter pass): item indices into pts, or, own non-null, the points
+  uint32_t* cand;
+  float4* own;
   float4* pts;         // n_items: collision point of each item, minus p0 (w: the item index's
                        // bits; stored by the count pass)
   int* status;
@@ -131,6 +133,8 @@ struct GridView {
   const float4* pts;     // the items' collision points (minus p0)
   int G;
   float origin, inv_h;
+  const float4* own = nullptr;  // batched steps that do not prune: the entries' own points
+                                // (then cand is not read), else null
 };
 
 // A grid of one cell that every position up to 10^6 m from the start falls into, with a
@@ -279,20 +283,20 @@ struct BatchView {
 cudaError_t launch_batch_partition(const BatchView& v, int blocks, cudaStream_t s);
 cudaError_t launch_batch_count(const BatchView& v, int blocks, cudaStream_t s);
 cudaError_t launch_batch_scan(const BatchView& v, int blocks, cudaStream_t s);
-cudaError_t launch_batch_scatter(const BatchView& v, int blocks, cudaStream_t s);
+cudaError_t launch_batch_scatter(const BatchView& v, int blocks, bool own, cudaStream_t s);
 cudaError_t launch_batch_prune(const BatchView& v, int blocks, cudaStream_t s);
 // lanes 1 or 4; dynamic: take units from the work queue, else stride by the grid;
 // six: the one-lane kernel compiled for six resident CTAs per SM (fewer
 // registers) instead of five; samples_per_cta: the one-lane pass's CTA size
 // (64, 128 or 256; the items' partial rows were laid out for it); overlap: as
-// launch_rollout's
+// launch_rollout's; own: the items' entries are their points
 cudaError_t launch_batch_rollout(const BatchView& v, int lanes, int it, int blocks, int dynamic,
-                                 int six, int samples_per_cta, bool overlap, cudaStream_t s);
+                                 int six, int samples_per_cta, bool own, bool overlap, cudaStream_t s);
 cudaError_t launch_batch_update(const BatchView& v, int it, int blocks, cudaStream_t s);
 
 // Resident CTAs per SM: {partition, count, scan, scatter, prune} and {rollout with one
 // lane per sample, with four, update, rollout with one lane compiled for six,
-// one lane with 64 samples per CTA, one lane with 256}.
+// one lane with 64 samples per CTA, one lane with 256} (the smaller of the two entry forms').
 cudaError_t batch_grid_occupancy(int out[5]);
 cudaError_t batch_rollout_occupancy(int out[6], int T_max);
 

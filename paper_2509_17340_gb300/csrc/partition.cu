@@ -333,11 +333,12 @@ __global__ void __launch_bounds__(256) k_partition(PartitionArgs a, const PartTa
 // K2a / K2d: candidate lists.  For every collision point p (item i), every
 // cell whose box is closer to p than `reach` gets p: the count pass adds to
 // the cell's counter, the scatter pass writes the entry at start(cell) + its
-// fill ticket.  An entry is i (the
-// count pass stores p at pts[i]; the points, far fewer than the entries, stay in
-// L1).  A point carries its item index in w (bits of an int), so that ties between
-// equidistant points are broken by item, the collision set's order, whatever the
-// order of the entries within a cell, which depends on the atomics.
+// fill ticket.  An entry is i (4 bytes; the count pass stores p at pts[i]; the points,
+// far fewer than the entries, stay in L1), or, in batched steps that do not prune, p
+// itself (16 bytes; one load less per entry read, where many planners' points share
+// an SM's L1).  Either way a point carries its item index in w (bits of an int), so
+// that ties between equidistant points are broken by item, the collision set's order,
+// whatever the order of the entries within a cell, which depends on the atomics.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ bool cand_item(const CandArgs& a, int64_t it, float& px, float& py,
                                           float& pz) {
@@ -362,8 +363,9 @@ __device__ __forceinline__ float gap2(float v, float lo, float h) {
   return d * d;
 }
 
-// One warp per collision item; its lanes share the item's block of cells.
-template <bool kScatter>
+// One warp per collision item; its lanes share the item's block of cells.  kOwn: the
+// entries are the points themselves (fixed per launch, so a template argument).
+template <bool kScatter, bool kOwn = false>
 __device__ __forceinline__ void cand_task(const CandArgs& a, int64_t it, int lane) {
   const GridGeom& g = a.grid;
   const float r2 = g.reach * g.reach;
@@ -428,7 +430,10 @@ __device__ __forceinline__ void cand_task(const CandArgs& a, int64_t it, int lan
         if (c[b] < 0) continue;
         const int pos = base[b] + ticket[b];
         if (pos < g.cap) {
-          a.cand[pos] = (uint32_t)it;
+          if constexpr (kOwn)
+            a.own[pos] = make_float4(px, py, pz, __int_as_float((int)it));
+          else
+            a.cand[pos] = (uint32_t)it;
         } else {
           atomicOr(a.status, 2);
         }
@@ -1078,7 +1083,7 @@ __global__ void __launch_bounds__(256) k_b_partition(BatchView v) {
 // stretches of the fine partition).  kScatter: the scatter pass, else the count.
 constexpr int kTaskChunk = 4;
 
-template <bool kScatter>
+template <bool kScatter, bool kOwn = false>
 __device__ __forceinline__ void cand_tasks(const BatchView& v, const long long* s_pi, int n,
                                            long long w, long long nw, int lane) {
   const long long ni = s_pi[n];
@@ -1093,7 +1098,7 @@ __device__ __forceinline__ void cand_tasks(const BatchView& v, const long long* 
         while (t >= s_pi[it + 1]) ++it;
         a = v.items[it].ca;
       }
-      cand_task<kScatter>(a, t - s_pi[it], lane);
+      cand_task<kScatter, kOwn>(a, t - s_pi[it], lane);
     }
   }
 }
@@ -1147,6 +1152,7 @@ __global__ void __launch_bounds__(kScanThreads) k_b_scan(BatchView v) {
 // Scatter tasks (emptying the keys they read); then the cell ranges and the
 // keys of planners whose collision set is every kept point (read only by the
 // coarse pass, so emptied here).
+template <bool kOwn>
 __global__ void __launch_bounds__(256) k_b_scatter(BatchView v) {
   pdl_start();
   __shared__ long long s_pi[kBatchMax + 1], s_pc[kBatchMax + 1];
@@ -1154,7 +1160,7 @@ __global__ void __launch_bounds__(256) k_b_scatter(BatchView v) {
   load_prefix(s_pi, v.pre + kPreItems * (n + 1), n);
   load_prefix(s_pc, v.pre + kPreCells * (n + 1), n);
   __syncthreads();
-  cand_tasks<true>(v, s_pi, n, ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5,
+  cand_tasks<true, kOwn>(v, s_pi, n, ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5,
                    (long long)gridDim.x * (blockDim.x >> 5), threadIdx.x & 31);
   const long long total = s_pc[n];
   const long long stride = (long long)gridDim.x * blockDim.x;
@@ -1276,7 +1282,11 @@ cudaError_t batch_grid_occupancy(int out[5]) {
   if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out + 1, k_b_count, 256, 0);
   if (e == cudaSuccess)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out + 2, k_b_scan, kScanThreads, 0);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out + 3, k_b_scatter, 256, 0);
+  // of the two entry forms
+  int own = 0;
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out + 3, k_b_scatter<false>, 256, 0);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&own, k_b_scatter<true>, 256, 0);
+  if (own < out[3]) out[3] = own;
   if (e == cudaSuccess)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out + 4, k_b_prune, kPruneThreads, sizeof(PruneSmem));
   for (int i = 0; i < 5; ++i)
@@ -1297,8 +1307,8 @@ cudaError_t launch_batch_scan(const BatchView& v, int blocks, cudaStream_t s) {
   return launch_k(k_b_scan, dim3(blocks), dim3(kScanThreads), s, true, v);
 }
 
-cudaError_t launch_batch_scatter(const BatchView& v, int blocks, cudaStream_t s) {
-  return launch_k(k_b_scatter, dim3(blocks), dim3(256), s, true, v);
+cudaError_t launch_batch_scatter(const BatchView& v, int blocks, bool own, cudaStream_t s) {
+  return launch_k(own ? k_b_scatter<true> : k_b_scatter<false>, dim3(blocks), dim3(256), s, true, v);
 }
 
 cudaError_t launch_batch_prune(const BatchView& v, int blocks, cudaStream_t s) {

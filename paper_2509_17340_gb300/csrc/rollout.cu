@@ -42,7 +42,9 @@ struct CostSum {
 // kWarpLists: long candidate lists scanned by the whole warp (warp_split_min,
 // lists longer than a.list_thr), for every-point collision sets whose lists are not
 // pruned; the others keep the per-lane scan, compiled without that path.
-template <bool kParams, int kNT = NT, bool kWarpLists = false, bool kRestForm = kParams && !kWarpLists>
+// kOwn: the grid's entries are the points themselves (batched steps that do not prune).
+template <bool kParams, int kNT = NT, bool kWarpLists = false, bool kRestForm = kParams && !kWarpLists,
+          bool kOwn = false>
 __device__ __forceinline__ void rollout_unit(const RolloutArgs& a, int e, int b, uint32_t ctr3) {
   constexpr int kNW = kNT / 32;
   constexpr int kSW = kNT > kMaxT ? kNT : kMaxT;
@@ -151,7 +153,7 @@ __device__ __forceinline__ void rollout_unit(const RolloutArgs& a, int e, int b,
                           a.list_thr);
     } else {
       for (int i = 0; i < range_j.y; ++i)
-        d2 = fminf(d2, dist2_to(grid_point(a.grid, range_j.x + i), x.p[0], x.p[1], x.p[2]));
+        d2 = fminf(d2, dist2_to(grid_point_of<kOwn>(a.grid, range_j.x + i), x.p[0], x.p[1], x.p[2]));
     }
     // state terms at x_j against the guide at t = j dt
     const float gx = s_gd[3 * (j - 1)], gy = s_gd[3 * (j - 1) + 1], gz = s_gd[3 * (j - 1) + 2];
@@ -329,6 +331,8 @@ __device__ __forceinline__ SplitSmem split_layout(unsigned char* base, int T) {
   return m;
 }
 
+// kEither: the grid's entries may be the points themselves (grid_point).
+template <bool kEither>
 __device__ __forceinline__ void rollout_split_unit(const RolloutArgs& a, int e, int b,
                                                    uint32_t ctr3) {
   extern __shared__ __align__(16) unsigned char split_smem[];
@@ -454,7 +458,7 @@ __device__ __forceinline__ void rollout_split_unit(const RolloutArgs& a, int e, 
       const int n = r.y - first < kItem ? r.y - first : kItem;
       if (!AERO_CHECK(slot < kChunkQ && first >= 0 && n > 0 && r.x >= 0, kChkQuery)) continue;
       const float4 p = xa[slot];
-      const float d2 = scan_min<kItem>(a.grid, r.x + first, n, p.x, p.y, p.z, dmax2);
+      const float d2 = scan_min<kItem, kEither>(a.grid, r.x + first, n, p.x, p.y, p.z, dmax2);
       if (d2 < dmax2) atomicMin(m.d2 + slot, __float_as_int(d2));  // non-negative: int order
     }
     warps_sync<SWK, kWorkBar>();  // minima complete
@@ -593,9 +597,10 @@ __device__ __forceinline__ UpdSmem update_layout(unsigned char* base, int T, int
 
 // kThreads: the CTA's threads (128 in the update kernels, 256 in the split
 // Stage I pass).  smem: update_smem_bytes(T, kThreads / 32, refine) bytes of
-// dynamic shared memory (16-byte aligned).  The partials are read through L2
+// dynamic shared memory (16-byte aligned).  kEither: the grid's entries may be the points
+// themselves (grid_point).  The partials are read through L2
 // (ld.cg): in the split pass other CTAs of the same launch wrote them.
-template <int kThreads>
+template <int kThreads, bool kEither>
 __device__ __forceinline__ void update_unit(const UpdateArgs& a, int e, bool final_stage,
                                             unsigned char* smem) {
   constexpr int UT = kThreads;
@@ -736,7 +741,7 @@ __device__ __forceinline__ void update_unit(const UpdateArgs& a, int e, bool fin
   if (a.refine_steps > 0) {
     if (a.dbg_pre)
       for (int i = tid; i < 4 * T; i += UT) a.dbg_pre[(size_t)e * T * 4 + i] = s_u[i];
-    block_refine<UT>(s_u4, a.guides + (size_t)e * T * 3, T, a.x0, a.dyn, a.cost, a.grid, a.umin,
+    block_refine<UT, kEither>(s_u4, a.guides + (size_t)e * T * 3, T, a.x0, a.dyn, a.cost, a.grid, a.umin,
                      a.umax, a.refine_steps, a.refine_step, refine_layout(sm.refine, T, UT / 32));
     for (int i = tid; i < 4 * T; i += UT) un[i] = s_u[i];
     __syncthreads();
@@ -774,7 +779,7 @@ __device__ __forceinline__ void update_unit(const UpdateArgs& a, int e, bool fin
     const int n = r.y - first < kItem ? r.y - first : kItem;
     if (!AERO_CHECK(j < T && first >= 0 && n > 0 && r.x >= 0, kChkQuery)) continue;
     const float* X = s_x + (j + 1) * 10;
-    const float d2 = scan_min<kItem>(a.grid, r.x + first, n, X[0], X[1], X[2], dmax2);
+    const float d2 = scan_min<kItem, kEither>(a.grid, r.x + first, n, X[0], X[1], X[2], dmax2);
     if (d2 < dmax2) atomicMin(s_d2 + j, __float_as_int(d2));  // non-negative: int order
   }
   __syncthreads();
@@ -924,7 +929,7 @@ __global__ void __launch_bounds__(ST, 2) k_rollout_split(RolloutArgs a, UpdateAr
   const int lin = (int)blockIdx.x - w;
   const int e = warm ? 0 : lin / a.nb;
   if (!warm) {
-    rollout_split_unit(a, e, lin - e * a.nb, a.ctr3);
+    rollout_split_unit<false>(a, e, lin - e * a.nb, a.ctr3);
     __threadfence();  // this CTA's partials are visible before its ticket
     __syncthreads();
     if (threadIdx.x == 0) s_last_b = atomicAdd(ua.inst_counter + e, 1u) == (unsigned)(a.nb - 1);
@@ -938,7 +943,7 @@ __global__ void __launch_bounds__(ST, 2) k_rollout_split(RolloutArgs a, UpdateAr
   __syncthreads();
   if (warm) warm_setup(&s_ua, ua, 0, nullptr);
   extern __shared__ __align__(16) unsigned char fused_smem[];  // the split pass's, free again
-  update_unit<ST>(s_ua, e, s_ua.final_stage != 0, fused_smem);
+  update_unit<ST, false>(s_ua, e, s_ua.final_stage != 0, fused_smem);
 }
 
 // The single-planner update: one CTA of ST threads per instance (the split
@@ -974,7 +979,7 @@ __global__ void __launch_bounds__(ST) k_update(UpdateArgs a) {
     block_copy_param(&s_a, &a);
     __syncthreads();
     if (run == 0) warm_setup(&s_a, a, blockIdx.x, a.warm_grid);
-    update_unit<ST>(s_a, blockIdx.x, s_a.final_stage != 0, upd_smem);
+    update_unit<ST, false>(s_a, blockIdx.x, s_a.final_stage != 0, upd_smem);
     __syncthreads();  // s_a and the scratch free for the next run
   }
   // the last CTA to leave resets the count and the exit ticket (every CTA has
@@ -992,8 +997,11 @@ __global__ void __launch_bounds__(ST) k_update(UpdateArgs a) {
 // resets it), else units are strided by the grid.  Planners whose iteration
 // count is at most `it` skip their units.
 // ---------------------------------------------------------------------------
-// kNT: samples per CTA of the one-lane pass (the autotuner's choice).
-template <int kLanes, int kMinCtas, int kNT = NT>
+// kNT: samples per CTA of the one-lane pass (the autotuner's choice); kOwn: its
+// entries are the points themselves.  Every-point sets of 16 planners (E = 8, K = 1024,
+// T = 40, up to 10,000 points) take 1.49 ms with the points, 2.66 with item indices and
+// 1.63 with indices and pruned lists; P_f of 8 planners 374, 421 and 284 us.
+template <int kLanes, int kMinCtas, int kNT = NT, bool kOwn = false>
 __global__ void __launch_bounds__(kLanes == 4 ? ST : kNT, kMinCtas)
     k_b_rollout(BatchView v, int it, int dynamic) {
   pdl_start();
@@ -1030,9 +1038,9 @@ __global__ void __launch_bounds__(kLanes == 4 ? ST : kNT, kMinCtas)
       const long long l = u - s_pre[pos];
       const int e = (int)(l / s_a.nb), b = (int)(l % s_a.nb);
       if constexpr (kLanes == 1)
-        rollout_unit<false, kNT, false, (kMinCtas == 5 && kNT == NT)>(s_a, e, b, s_a.ctr3 | (uint32_t)it);
+        rollout_unit<false, kNT, false, (kMinCtas == 5 && kNT == NT), kOwn>(s_a, e, b, s_a.ctr3 | (uint32_t)it);
       else
-        rollout_split_unit(s_a, e, b, s_a.ctr3 | (uint32_t)it);
+        rollout_split_unit<true>(s_a, e, b, s_a.ctr3 | (uint32_t)it);
     }
     if (!dynamic) u += gridDim.x;
     __syncthreads();  // the unit's shared memory is free again
@@ -1067,7 +1075,7 @@ __global__ void __launch_bounds__(UT) k_b_update(BatchView v, int it) {
       __syncthreads();
       cur = item;
     }
-    if (it < s_iters) update_unit<UT>(s_a, (int)(u - s_pre[item]), it == s_iters - 1, upd_smem);
+    if (it < s_iters) update_unit<UT, true>(s_a, (int)(u - s_pre[item]), it == s_iters - 1, upd_smem);
     __syncthreads();
   }
 }
@@ -1166,32 +1174,40 @@ cudaError_t split_carveout(int T) {
 
 cudaError_t batch_rollout_occupancy(int out[6], int T_max) {
   cudaError_t e = split_attributes();
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out + 0, k_b_rollout<1, 5>, NT, 0);
+  // one lane per sample: the smaller of the two entry forms
+  auto one_lane = [&](int k, auto* indices, auto* own, int threads) {
+    int a = 0, b = 0;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&a, indices, threads, 0);
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&b, own, threads, 0);
+    out[k] = a < b ? a : b;
+  };
+  one_lane(0, k_b_rollout<1, 5>, k_b_rollout<1, 5, NT, true>, NT);
+  one_lane(3, k_b_rollout<1, 6>, k_b_rollout<1, 6, NT, true>, NT);
+  one_lane(4, k_b_rollout<1, 12, 64>, k_b_rollout<1, 12, 64, true>, 64);
+  one_lane(5, k_b_rollout<1, 3, 256>, k_b_rollout<1, 3, 256, true>, 256);
   if (e == cudaSuccess)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out + 1, k_b_rollout<4, 2>, ST,
                                                       split_smem_bytes(T_max));
   if (e == cudaSuccess)
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out + 2, k_b_update, UT,
                                                       update_smem_bytes(T_max, UT / 32, true));
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out + 3, k_b_rollout<1, 6>, NT, 0);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out + 4, k_b_rollout<1, 12, 64>, 64, 0);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(out + 5, k_b_rollout<1, 3, 256>, 256, 0);
   for (int i = 0; i < 6; ++i)
     if (out[i] < 1) out[i] = 1;
   return e;
 }
 
 cudaError_t launch_batch_rollout(const BatchView& v, int lanes, int it, int blocks, int dynamic,
-                                 int six, int samples_per_cta, bool overlap, cudaStream_t s) {
+                                 int six, int samples_per_cta, bool own, bool overlap, cudaStream_t s) {
   if (lanes == 4)
     return launch_ks(k_b_rollout<4, 2>, dim3(blocks), dim3(ST), split_smem_bytes(v.T_max), s, true, v,
                      it, dynamic);
-  if (samples_per_cta == 64)
-    return launch_k(k_b_rollout<1, 12, 64>, dim3(blocks), dim3(64), s, overlap, v, it, dynamic);
-  if (samples_per_cta == 256)
-    return launch_k(k_b_rollout<1, 3, 256>, dim3(blocks), dim3(256), s, overlap, v, it, dynamic);
-  if (six) return launch_k(k_b_rollout<1, 6>, dim3(blocks), dim3(NT), s, overlap, v, it, dynamic);
-  return launch_k(k_b_rollout<1, 5>, dim3(blocks), dim3(NT), s, overlap, v, it, dynamic);
+  auto one_lane = [&](auto* indices, auto* points, int threads) {
+    return launch_k(own ? points : indices, dim3(blocks), dim3(threads), s, overlap, v, it, dynamic);
+  };
+  if (samples_per_cta == 64) return one_lane(k_b_rollout<1, 12, 64>, k_b_rollout<1, 12, 64, true>, 64);
+  if (samples_per_cta == 256) return one_lane(k_b_rollout<1, 3, 256>, k_b_rollout<1, 3, 256, true>, 256);
+  if (six) return one_lane(k_b_rollout<1, 6>, k_b_rollout<1, 6, NT, true>, NT);
+  return one_lane(k_b_rollout<1, 5>, k_b_rollout<1, 5, NT, true>, NT);
 }
 
 cudaError_t launch_batch_update(const BatchView& v, int it, int blocks, cudaStream_t s) {
