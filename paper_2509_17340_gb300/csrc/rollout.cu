@@ -40,8 +40,8 @@ struct CostSum {
 // (step_id << 8) | iteration.  kParams: the arguments are
 // kernel parameters (a single planner's step), else in shared memory.
 // kWarpLists: long candidate lists scanned by the whole warp (warp_split_min,
-// lists longer than a.list_thr), for every-point collision sets whose lists are not
-// pruned; the others keep the per-lane scan, compiled without that path.
+// lists longer than a.list_thr), for every-point collision sets; the others keep the
+// per-lane scan, compiled without that path.
 // kOwn: the grid's entries are the points themselves (batched steps that do not prune).
 template <bool kParams, int kNT = NT, bool kWarpLists = false, bool kRestForm = kParams && !kWarpLists,
           bool kOwn = false>
