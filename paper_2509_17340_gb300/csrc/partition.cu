@@ -143,6 +143,10 @@ constexpr int kOutside = -1;    // cone_of: outside the range or the elevation s
 // with cones of 1.4 to 3 degrees, take the exact predicates.  Ten million points:
 // the launch 73.3 -> 60.6 us (169 warp instructions per 32 points, issue slots 73%
 // busy; its 120 MB take 18 us at the copy rate).
+//
+// kUnbounded: the range bound's square is infinite (a.unbounded), compiled apart: the
+// test for it on every point outside made the same launch 62.5 -> 65.9 us.
+template <bool kUnbounded>
 __device__ __forceinline__ int cone_of(const PartitionArgs& a, const SmemTables& st, float3 pt,
                                        float* r2_out) {
   const float dx = sub(pt.x, a.p0[0]), dy = sub(pt.y, a.p0[1]), dz = sub(pt.z, a.p0[2]);
@@ -153,8 +157,8 @@ __device__ __forceinline__ int cone_of(const PartitionArgs& a, const SmemTables&
   // a non-finite coordinate makes every component of b infinite or NaN, and r2 above the
   // (finite) bound
   if (!(r2 > 0.0f && r2 <= a.rmax2)) {
-    if (!(isfinite(pt.x) && isfinite(pt.y) && isfinite(pt.z))) return kNonFinite;
-    if (!(a.unbounded && r2 == INFINITY)) return kOutside;
+    const bool finite = isfinite(pt.x) && isfinite(pt.y) && isfinite(pt.z);
+    if (!(kUnbounded && finite && r2 == INFINITY)) return finite ? kOutside : kNonFinite;
   }
   const float ga = (atan2_guess(b[1], b[0]) + 3.141592654f) * a.az_scale;
   const float ge = (atan2_guess(b[2], fast_sqrt(rxy2)) - a.el_lo) * a.el_inv;
@@ -184,10 +188,11 @@ __device__ __forceinline__ unsigned long long cone_key(float r2, uint32_t i) {
 
 // Point i at (px, py, pz).  Returns 0 for a non-finite point, 1 for a point
 // outside the partition's range or elevation span, 2 for a kept point.
+template <bool kUnbounded>
 __device__ __forceinline__ int partition_point(const PartitionArgs& a, const SmemTables& st,
                                                int64_t i, float3 pt) {
   float r2 = 0.0f;
-  const int c = cone_of(a, st, pt, &r2);
+  const int c = cone_of<kUnbounded>(a, st, pt, &r2);
   if (c >= 0) {
     const unsigned long long key = cone_key(r2, (uint32_t)i);
     // dense clouds: a key at or above the cone's current minimum cannot
@@ -203,6 +208,7 @@ __device__ __forceinline__ int partition_point(const PartitionArgs& a, const Sme
 // Points 4 g .. 4 g + 3 (a 16-byte aligned cloud: three float4 loads).  The
 // four cones are found first and their keys read together, so that the four
 // reads of the current minima are in flight at once.
+template <bool kUnbounded>
 __device__ __forceinline__ void partition_group(const PartitionArgs& a, const SmemTables& st,
                                                 int64_t g, float4 v0, float4 v1, float4 v2,
                                                 int& nf, int& kept) {
@@ -214,7 +220,7 @@ __device__ __forceinline__ void partition_group(const PartitionArgs& a, const Sm
 #pragma unroll
   for (int j = 0; j < 4; ++j) {
     float r2 = 0.0f;
-    c[j] = cone_of(a, st, pt[j], &r2);
+    c[j] = cone_of<kUnbounded>(a, st, pt[j], &r2);
     key[j] = cone_key(r2, i0 + j);
   }
   unsigned long long cur[4];
@@ -258,8 +264,9 @@ constexpr int kPartBlocksPerSm = 16;
 
 
 // kGroups: four points per thread (launched for clouds of at least
-// kPartVecMin points whose buffers are 16-byte aligned), else one.
-template <bool kGroups>
+// kPartVecMin points whose buffers are 16-byte aligned), else one.  kUnbounded: as
+// cone_of's.
+template <bool kGroups, bool kUnbounded>
 __global__ void __launch_bounds__(256) k_partition(PartitionArgs a, const PartTables* __restrict__ t) {
   pdl_start();
   __shared__ SmemTables st;
@@ -293,7 +300,7 @@ __global__ void __launch_bounds__(256) k_partition(PartitionArgs a, const PartTa
         d[1] = w1;
         d[2] = w2;
       }
-      partition_group(a, st, g, w0, w1, w2, nf, kept);
+      partition_group<kUnbounded>(a, st, g, w0, w1, w2, nf, kept);
     }
     // the last n mod 4 points
     const int64_t i = 4 * ng + tid;
@@ -304,7 +311,7 @@ __global__ void __launch_bounds__(256) k_partition(PartitionArgs a, const PartTa
         a.copy_to[3 * i + 1] = pt.y;
         a.copy_to[3 * i + 2] = pt.z;
       }
-      const int r = partition_point(a, st, i, pt);
+      const int r = partition_point<kUnbounded>(a, st, i, pt);
       nf += r == 0;
       kept += r == 2;
     }
@@ -320,7 +327,7 @@ __global__ void __launch_bounds__(256) k_partition(PartitionArgs a, const PartTa
         a.copy_to[3 * i + 1] = pt.y;
         a.copy_to[3 * i + 2] = pt.z;
       }
-      const int r = partition_point(a, st, i, pt);
+      const int r = partition_point<kUnbounded>(a, st, i, pt);
       nf += r == 0;
       kept += r == 2;
       if (i + stride < a.n) pt = cloud_point(a, i + stride);
@@ -1070,7 +1077,9 @@ __global__ void __launch_bounds__(256) k_b_partition(BatchView v) {
     int nf = 0, kept = 0;
     for (int r = threadIdx.x; r < kPartChunk; r += blockDim.x)
       if (base + r < s_pa.n) {
-        const int c = partition_point(s_pa, st, base + r, cloud_point(s_pa, base + r));
+        const float3 pt = cloud_point(s_pa, base + r);
+        const int c = s_pa.unbounded ? partition_point<true>(s_pa, st, base + r, pt)
+                                     : partition_point<false>(s_pa, st, base + r, pt);
         nf += c == 0;
         kept += c == 2;
       }
@@ -1230,9 +1239,10 @@ cudaError_t launch_partition(const PartitionArgs& a, const PartTables* t, cudaSt
   const uintptr_t bits = reinterpret_cast<uintptr_t>(a.cloud) |
                          reinterpret_cast<uintptr_t>(a.copy_to) |
                          reinterpret_cast<uintptr_t>(a.item_flag);
-  if (a.n >= kPartVecMin && (bits & 15u) == 0)
-    return launch_k(k_partition<true>, dim3(partition_blocks(a.n)), dim3(256), s, true, a, t);
-  return launch_k(k_partition<false>, dim3(partition_blocks(a.n)), dim3(256), s, true, a, t);
+  const bool groups = a.n >= kPartVecMin && (bits & 15u) == 0;
+  auto* const kernel = groups ? (a.unbounded ? k_partition<true, true> : k_partition<true, false>)
+                              : (a.unbounded ? k_partition<false, true> : k_partition<false, false>);
+  return launch_k(kernel, dim3(partition_blocks(a.n)), dim3(256), s, true, a, t);
 }
 
 cudaError_t launch_grid_count(const CandArgs& ca, const GuideArgs& ga, cudaStream_t s) {
