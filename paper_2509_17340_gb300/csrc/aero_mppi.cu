@@ -203,13 +203,19 @@ constexpr int kFineDup = 216, kCoarseDup = 27;
 // atomic minimum: in dense clouds most points cannot lower their cone's key
 constexpr int64_t kPartFilterPointsPerCone = 32;
 // lists longer than this are scanned by the whole warp in the one-lane pass
-// when every kept point is the collision set: whole lists, and pruned ones (shorter, so
-// fewer are worth the warp's turn; of 8, 16 and 32 it is the best or within 5%)
-constexpr int kWarpListThreshold = 8, kWarpListPruned = 16;
-// when lists are pruned (prunes_lists)
-constexpr int64_t kPruneStepsPerPoint = 14, kPruneSteps = 12000000;
+// when every kept point is the collision set: whole lists, and lists that may be pruned
+// (shorter, so fewer are worth the warp's turn: large clutter with every point 1.584,
+// 1.492, 1.435 and 1.512 ms a step for 16, 32, 64 and 128, 1.504 without; nine other
+// steps within 4% from 16 to 64)
+constexpr int kWarpListThreshold = 8, kWarpListPruned = 64;
+// when a single planner's lists may be pruned (prunes_lists)
+constexpr int64_t kPruneRawSteps = 200000, kPruneStepsPerPoint = 14;
+constexpr int64_t kPruneOneLaneSteps = 2000000, kPruneSteps = 12000000;
 constexpr int64_t kPruneDenseSteps = 100000, kPruneDensePointsPerCone = 16;
-constexpr int kPruneDenseEntries = 131072, kPruneDenseEntriesPerCell = 2;
+// and are: from how many entries met by the samples (sample-steps x mean length of the
+// lists at the probe's positions), kPruneMet and kPruneMetPerEntry for every entry of all
+// lists; {split pass, one-lane pass}
+constexpr float kPruneMet[2] = {2.5e6f, 1.5e6f}, kPruneMetPerEntry[2] = {5.0f, 4.0f};
 constexpr int64_t kPruneBatchSteps = 400000;
 
 int cuda_fail(cudaError_t e) {
@@ -613,20 +619,54 @@ void make_step_args(aero_planner* pl, const aero_state_t* x0, const float* cloud
   ra.done = ua.done;
 }
 
-// Whether a single planner's step prunes its candidate lists (k_grid_prune), and from
-// how many entries in all.  Pruning takes time by the entries, what it saves goes by
-// the sample-steps.  Every kept point: 178,000 points cost 320 us and save 0.12 ns and
-// more per sample-step, so from 14 sample-steps per point on.  P_f of a sparse
-// scene (555,000 entries, 36 us): 0.004 ns, so from 12 M sample-steps on.  P_f of a
-// dense one (0.2 to 0.8 ns) from 100,000 on; that it is dense is likely where the
-// cloud has 16 points per cone, and decided on the device by two entries per cell.
-bool prunes_lists(const aero_params_t& p, int64_t n, const StepArgs& a, int& min_total) {
+// Whether a single planner's step may prune its candidate lists: a rule on the host for
+// the steps in which pruning can pay, then, on the device, the list probe
+// (probe_lists).  Pruning takes time by the entries (36 us for 0.6 M, 20 to 50 for 0.25 M
+// in long lists) and saves by the entries that the samples meet, 1 to 10 ps for each:
+// the probe's line lies where the two sides of 114 steps (scenes, sizes, both sets)
+// cross.  Flight cycle, 16 scenes: 85 to 547 us whole, 86 to
+// 263 by the probe, 100 to 249 always pruned; 200,000 points of a clutter seen from
+// afar: 54 whole, 57 by the probe, 72 pruned; 100,000 of ten pillars off the path, the
+// every-point set: 189, 177 and 331; large clutter, six scenes: 383 to 536 whole, 355 to
+// 382 by the probe.  A probe that leaves the lists whole costs 2 to 5 us, so the host
+// leaves out smaller steps: every kept point below 200,000 sample-steps or 14 per point,
+// P_f of the one-lane pass below 2 M (169 whole and 172 probed at 1.6 M; 242 whole and 146
+// at 3 M) unless the cloud has 16 points per cone, as dense maps and accumulated
+// sweeps close by do.
+bool prunes_lists(const aero_params_t& p, int64_t n, const StepArgs& a) {
   const int64_t steps = (int64_t)p.E * p.K * p.T * p.iters;
-  min_total = 0;
-  if (a.raw) return steps >= kPruneStepsPerPoint * n;
-  if (steps >= kPruneSteps) return true;
-  min_total = std::max(kPruneDenseEntries, kPruneDenseEntriesPerCell * a.gcells);
-  return steps >= kPruneDenseSteps && n >= kPruneDensePointsPerCone * a.ncell;
+  if (a.raw) return steps >= kPruneRawSteps && steps >= kPruneStepsPerPoint * n;
+  return steps >= (a.lanes == 1 ? kPruneOneLaneSteps : kPruneSteps) ||
+         (steps >= kPruneDenseSteps && n >= kPruneDensePointsPerCone * a.ncell);
+}
+
+// Whether the probe decides: not for P_f from 12 M sample-steps on, where every scene
+// measured gained (21 to 330 us of 380 to 750).
+bool probes_lists(const aero_params_t& p, const StepArgs& a) {
+  return a.raw || (int64_t)p.E * p.K * p.T * p.iters < kPruneSteps;
+}
+
+ProbeArgs make_probe(aero_planner* pl, const aero_params_t& p, const StepArgs& a) {
+  ProbeArgs b;
+  b.blocks = kProbeBlocks;
+  b.E = p.E;
+  b.K = p.K;
+  b.T = p.T;
+  b.per = (p.T + kProbeSteps - 1) / kProbeSteps;
+  b.steps = (p.T + b.per - 1) / b.per;
+  std::memcpy(b.x0, a.ra.x0, sizeof(b.x0));
+  b.dyn = a.ra.dyn;
+  for (int c = 0; c < 4; ++c) {
+    b.sigma[c] = a.ra.sigma[c];
+    b.umin[c] = a.ra.umin[c];
+    b.umax[c] = a.ra.umax[c];
+  }
+  b.key0 = a.ra.key0;
+  b.key1 = a.ra.key1;
+  b.ctr3 = a.ra.ctr3;
+  b.u_nom = a.ra.u_nom;
+  b.sum = reinterpret_cast<int*>(pl->counter + kProbeWord);
+  return b;
 }
 
 // The planner's state after a step has been enqueued.
@@ -731,18 +771,23 @@ int enqueue_step(aero_planner* pl, const aero_state_t* x0, const float* cloud, i
                             pl->tile_off, a.gcells + 1, a.ntiles, nullptr, a.ga, pl->d_tab, s)) !=
       cudaSuccess)
     return cuda_fail(e);
+  const bool prune = prunes_lists(p, n, a);
+  ProbeArgs probe;
+  if (prune && probes_lists(p, a)) probe = make_probe(pl, p, a);
   if ((e = launch_grid_scatter(a.ca, pl->grid_range, a.gcells, pl->tile_sum, pl->tile_off,
-                               a.ntiles, s)) != cudaSuccess)
+                               a.ntiles, probe, s)) != cudaSuccess)
     return cuda_fail(e);
-  int min_total = 0;
-  const bool prune = prunes_lists(p, n, a, min_total);
   // every kept point as the collision set: lists of tens to hundreds of entries, uneven
   // across a warp's queries, also once pruned (60,000 points of a forest, 2 M sample-steps,
-  // whole step: 2437 us whole, 3064 pruned, 1166 pruned and scanned by the warp)
+  // whole step: 2437 us whole, 3064 pruned, 1153 pruned and scanned by the warp)
   a.ra.list_thr = !a.raw ? 0 : prune ? kWarpListPruned : kWarpListThreshold;
   if (prune) {
+    // the probe's sum at which pruning pays
+    const float scale = 32.0f * kProbeBlocks * (float)probe.steps / (float)((int64_t)p.E * p.K * p.T * p.iters);
+    const int one = a.lanes == 1 ? 1 : 0;
     const PruneArgs pr{pl->cand, pl->cand_pts, pl->grid_range, (int)a.n_items, a.gcells, 0,
-                       min_total > 0 ? pl->tile_off + a.ntiles : nullptr, min_total, a.grid};
+                       pl->tile_off + a.ntiles, probe.blocks > 0 ? probe.sum : nullptr, kPruneMet[one] * scale,
+                       kPruneMetPerEntry[one] * scale, a.grid};
     if ((e = launch_grid_prune(pr, s)) != cudaSuccess) return cuda_fail(e);
     if (prof) ++prof->launches[AERO_STAGE_GRID];
   }

@@ -17,8 +17,12 @@ constexpr int kMaxE = 64;
 // [0] selection ticket, [1], [2] grid counters, [3, 3 + kMaxE) the split pass's
 // instance tickets, then the one-lane pass's finished-CTA count and the update
 // launch's exit ticket
-constexpr int kCounterWords = 5 + kMaxE;
+// then the list probe's sums
+constexpr int kProbeBlocks = 8;  // blocks of the list probe, 32 samples each
+constexpr int kProbeSteps = 16;  // its integration steps, at most
 constexpr int kDoneWord = 3 + kMaxE;
+constexpr int kProbeWord = 5 + kMaxE;
+constexpr int kCounterWords = kProbeWord + kProbeBlocks;
 constexpr int kMaxT = 128;
 constexpr int kGridMax = 96;         // collision-grid cells per axis, at most
 constexpr int kGridCellsMax = kGridMax * kGridMax * kGridMax;
@@ -101,8 +105,11 @@ struct PruneArgs {
   int items;               // collision items
   int ncells;
   int runs;                // runs of cells per unit (set by the launch)
-  const int* total;        // entries of all lists, or null; below min_total the lists stay whole
-  int min_total;
+  // The lists stay whole where the probe's sums add up to less than need + need_entry x
+  // the entries of all lists (probe null: always pruned).
+  const int* total;
+  const int* probe;
+  float need, need_entry;
   GridGeom grid;
 };
 
@@ -156,6 +163,19 @@ struct CostParams {
 
 struct DynParams {
   float dt, inv_mass, g;
+};
+
+// The list probe: kProbeBlocks x 32 coarse sample trajectories (`steps` integration
+// steps of `per` rollout steps each), whose positions' list lengths are summed.
+struct ProbeArgs {
+  int blocks = 0;          // kProbeBlocks, or 0: no probe
+  int E = 0, K = 0, T = 0, steps = 0, per = 0;
+  float x0[10] = {};
+  DynParams dyn{};
+  float sigma[4] = {}, umin[4] = {}, umax[4] = {};
+  uint32_t key0 = 0, key1 = 0, ctr3 = 0;
+  const float* u_nom = nullptr;  // E x T x 4
+  int* sum = nullptr;      // one word per block
 };
 
 struct RolloutArgs {
@@ -312,10 +332,10 @@ cudaError_t launch_grid_count(const CandArgs& ca, const GuideArgs& ga, cudaStrea
 cudaError_t launch_grid_scan(int* count, int* fill, int* local, int* tile_sum, int* tile_off,
                              int ncells, int ntiles, unsigned int* counter, const GuideArgs& ga,
                              const PartTables* t, cudaStream_t s);
-// scatter + cell ranges; the tile offsets are computed here from the tile
-// totals of the scan launch (and written to tile_off)
+// scatter + cell ranges + the list probe; the tile offsets are computed here from the
+// tile totals of the scan launch (and written to tile_off)
 cudaError_t launch_grid_scatter(const CandArgs& ca, int2* range, int ncells, const int* tile_sum,
-                                int* tile_off, int ntiles, cudaStream_t s);
+                                int* tile_off, int ntiles, const ProbeArgs& probe, cudaStream_t s);
 // the lists pruned to the entries that can be a query's nearest, the ranges with them
 cudaError_t launch_grid_prune(PruneArgs a, cudaStream_t s);
 cudaError_t prune_attributes();  // its shared-memory limit (set by split_attributes)

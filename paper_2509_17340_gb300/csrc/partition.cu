@@ -719,14 +719,82 @@ __device__ __forceinline__ void range_cell(const int* local, const int* tile_off
   range[c] = AERO_CHECK(s >= 0 && e >= s, kChkRange) ? make_int2(s, e - s) : make_int2(0, 0);
 }
 
+// The list probe: what pruning saves goes by the lists that Stage I's samples meet, and
+// those are not the totals: dense ground or pillars away from the trajectories have long
+// lists that no query scans.  A block takes 32 samples (the instances in turn; a sample's
+// noise is drawn once for `per` steps together, its variance divided by them) through a
+// coarse semi-implicit integration of the model and adds up the list lengths at its
+// positions.  Its time (about 2 us) is the chain of at most kProbeSteps short steps on one
+// warp: the controls before it and the lengths after it are shared out over all warps,
+// and the scatter's blocks run beside it.
+struct ProbeSmem {
+  float4 u[kProbeSteps][32];
+  int cell[kProbeSteps][32];
+  int sum;
+};
+
+__device__ __forceinline__ void probe_lists(const ProbeArgs& p, const GridGeom& g, const int* local,
+                                            const int* s_off, int block, ProbeSmem& sm) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, warps = blockDim.x >> 5;
+  const int t = 32 * block + lane, e = t % p.E, k = t / p.E % p.K;
+  const float ns = rsqrtf((float)p.per);
+  const float4 sigma = make_float4(ns * p.sigma[0], ns * p.sigma[1], ns * p.sigma[2], ns * p.sigma[3]);
+  const float4* un = reinterpret_cast<const float4*>(p.u_nom) + (size_t)e * p.T;
+  if (threadIdx.x == 0) sm.sum = 0;
+  for (int j = wid; j < p.steps; j += warps) {
+    const float4 n = __ldcg(un + min(j * p.per + p.per / 2, p.T - 1));
+    const float4 d = noise_delta(k, j, e, p.ctr3, p.key0, p.key1, sigma);
+    sm.u[j][lane] = make_float4(fminf(fmaxf(n.x + d.x, p.umin[0]), p.umax[0]),
+                                fminf(fmaxf(n.y + d.y, p.umin[1]), p.umax[1]),
+                                fminf(fmaxf(n.z + d.z, p.umin[2]), p.umax[2]),
+                                fminf(fmaxf(n.w + d.w, p.umin[3]), p.umax[3]));
+  }
+  __syncthreads();
+  if (wid == 0) {
+    const float h = p.dyn.dt * (float)p.per, h2 = 0.5f * h;
+    float px = p.x0[0], py = p.x0[1], pz = p.x0[2], vx = p.x0[7], vy = p.x0[8], vz = p.x0[9];
+    float4 q = make_float4(p.x0[3], p.x0[4], p.x0[5], p.x0[6]);
+    for (int j = 0; j < p.steps; ++j) {
+      const float4 u = sm.u[j][lane];
+      const float4 y = quat_mul4(q, make_float4(1.0f, h2 * u.y, h2 * u.z, h2 * u.w));
+      const float inv = fast_rsqrt(y.x * y.x + y.y * y.y + y.z * y.z + y.w * y.w);
+      q = make_float4(y.x * inv, y.y * inv, y.z * inv, y.w * inv);
+      float rx, ry, rz;
+      r_e3(q.x, q.y, q.z, q.w, rx, ry, rz);
+      const float f = h * u.x * p.dyn.inv_mass;
+      vx += f * rx;
+      vy += f * ry;
+      vz += f * rz - h * p.dyn.g;
+      px += h * vx;
+      py += h * vy;
+      pz += h * vz;
+      const int ix = __float2int_rd((px - g.origin) * g.inv_h), iy = __float2int_rd((py - g.origin) * g.inv_h),
+                iz = __float2int_rd((pz - g.origin) * g.inv_h);
+      const bool in = (unsigned)ix < (unsigned)g.G && (unsigned)iy < (unsigned)g.G && (unsigned)iz < (unsigned)g.G;
+      sm.cell[j][lane] = in ? (iz * g.G + iy) * g.G + ix : -1;
+    }
+  }
+  __syncthreads();
+  int sum = 0;
+  for (int j = wid; j < p.steps; j += warps) {
+    const int c = sm.cell[j][lane];
+    if (c >= 0)
+      sum += local[c + 1] + s_off[(c + 1) >> kScanTileShift] - local[c] - s_off[c >> kScanTileShift];
+  }
+  sum = __reduce_add_sync(0xffffffffu, sum);
+  if (lane == 0) atomicAdd(&sm.sum, sum);
+  __syncthreads();
+  if (threadIdx.x == 0) p.sum[block] = sm.sum;
+}
+
 // K2c: the scatter pass and, in the remaining blocks, the {start, count} of
-// every cell (which needs only the scan).  Every block first turns the scan's
-// tile totals into tile offsets in shared memory (at most kMaxTiles of them);
-// block 0 also stores them.
+// every cell (which needs only the scan) and the list probe.  Every block first turns
+// the scan's tile totals into tile offsets in shared memory (at most kMaxTiles of
+// them); block 0 also stores them.
 __global__ void __launch_bounds__(256) k_grid_scatter(CandArgs ca, int scatter_blocks,
                                                       int2* __restrict__ range, int ncells,
                                                       const int* tile_sum, int* tile_off,
-                                                      int ntiles) {
+                                                      int ntiles, ProbeArgs probe) {
   pdl_start();
   __shared__ int s_off[kMaxTiles + 1];
   __shared__ int s_warp[32];
@@ -747,15 +815,21 @@ __global__ void __launch_bounds__(256) k_grid_scatter(CandArgs ca, int scatter_b
   __syncthreads();
   if (blockIdx.x == 0)
     for (int i = threadIdx.x; i <= ntiles; i += blockDim.x) tile_off[i] = s_off[i];
-  if ((int)blockIdx.x < scatter_blocks) {
-    CandArgs a = ca;
-    a.tile_off = s_off;
-    cand_pass<true>(a, blockIdx.x, scatter_blocks);
+  // the probe's blocks first: theirs is the longest chain
+  if ((int)blockIdx.x < probe.blocks) {
+    extern __shared__ __align__(16) unsigned char probe_smem[];
+    probe_lists(probe, ca.grid, ca.local, s_off, blockIdx.x, *reinterpret_cast<ProbeSmem*>(probe_smem));
     return;
   }
-  const int nrb = (int)gridDim.x - scatter_blocks;
-  for (int c = (blockIdx.x - scatter_blocks) * blockDim.x + threadIdx.x; c < ncells;
-       c += nrb * blockDim.x)
+  const int b = (int)blockIdx.x - probe.blocks;
+  if (b < scatter_blocks) {
+    CandArgs a = ca;
+    a.tile_off = s_off;
+    cand_pass<true>(a, b, scatter_blocks);
+    return;
+  }
+  const int nrb = (int)gridDim.x - probe.blocks - scatter_blocks;
+  for (int c = (b - scatter_blocks) * blockDim.x + threadIdx.x; c < ncells; c += nrb * blockDim.x)
     range_cell(ca.local, s_off, ca.grid.cap, range, c);
 }
 
@@ -1026,7 +1100,12 @@ __device__ void prune_cells(const PruneArgs& a, PruneSmem& sm, int c, int2 r) {
 
 __global__ void __launch_bounds__(kPruneThreads) k_grid_prune(PruneArgs a) {
   pdl_start();
-  if (a.total && __ldg(a.total) < a.min_total) return;
+  if (a.probe) {
+    int sum = 0;
+#pragma unroll
+    for (int i = 0; i < kProbeBlocks; ++i) sum += __ldg(a.probe + i);
+    if ((float)sum < a.need + a.need_entry * (float)__ldg(a.total)) return;
+  }
   extern __shared__ __align__(16) unsigned char prune_smem[];
   const int c = prune_cell_of(a.runs, a.ncells, blockIdx.x, gridDim.x);
   prune_cells(a, *reinterpret_cast<PruneSmem*>(prune_smem), c, c >= 0 ? a.range[c] : make_int2(0, 0));
@@ -1214,7 +1293,7 @@ __global__ void __launch_bounds__(kPruneThreads) k_b_prune(BatchView v) {
     const int2 ru = r;
     fetch(u + gridDim.x);  // the next unit's ranges are on their way meanwhile
     const PruneArgs a{bi->ca.cand, bi->ca.pts, bi->range, (int)bi->ca.n_items, bi->gcells,
-                      kPruneCells / kPruneRun, nullptr, 0, bi->ca.grid};
+                      kPruneCells / kPruneRun, nullptr, nullptr, 0.0f, 0.0f, bi->ca.grid};
     prune_cells(a, *reinterpret_cast<PruneSmem*>(prune_smem), cu, ru);
     __syncthreads();  // the unit's shared memory is free again
   }
@@ -1261,12 +1340,13 @@ cudaError_t launch_grid_scan(int* count, int* fill, int* local, int* tile_sum, i
 }
 
 cudaError_t launch_grid_scatter(const CandArgs& ca, int2* range, int ncells, const int* tile_sum,
-                                int* tile_off, int ntiles, cudaStream_t s) {
+                                int* tile_off, int ntiles, const ProbeArgs& probe, cudaStream_t s) {
   const int sms = device_sms();
   const int scatter_blocks = ca.n_items > 0 ? blocks_for(ca.n_items * 32, 256, 4 * sms) : 0;
   const int range_blocks = blocks_for(ncells, 256, 2 * sms);
-  return launch_k(k_grid_scatter, dim3(scatter_blocks + range_blocks), dim3(256), s, true, ca,
-                  scatter_blocks, range, ncells, tile_sum, tile_off, ntiles);
+  return launch_ks(k_grid_scatter, dim3(probe.blocks + scatter_blocks + range_blocks), dim3(256),
+                   probe.blocks > 0 ? sizeof(ProbeSmem) : 0, s, true, ca, scatter_blocks, range, ncells,
+                   tile_sum, tile_off, ntiles, probe);
 }
 
 cudaError_t launch_grid_prune(PruneArgs a, cudaStream_t s) {

@@ -27,18 +27,18 @@ def test_tied_seeds(aero, pitch):  # noqa: F811
     w.cloud = p[rng.permutation(len(p))]
     w.v0 = np.array([1.6, 1.6, 1.6], np.float32)
     P = w.params
-    K = 32 * (14 * len(p) // (32 * 20) + 1)     # sample-steps from which such a set is pruned
+    K, D = 1 << 14, 1024      # sample-steps that meet enough entries for such a set to be pruned
     P.update(E=1, M_h=1, M_v=1, K=K, T=20, r_max=10.0, collision_set=1, lanes_per_sample=4,
-             debug_samples=K, sigma=[2.0, 1.5, 1.5, 1.5])
+             debug_samples=D, sigma=[2.0, 1.5, 1.5, 1.5])
     pl = aero.Planner(E_max=1, K_max=K, T_max=20, fine_cells_max=P["fine_az"] * P["fine_el"],
-                      n_points_max=len(p), debug_samples_max=K)
+                      n_points_max=len(p), debug_samples_max=D)
     try:
         run_gpu(aero, pl, w, P, w.hover_nominal())
-        x = pl.debug("SAMPLE_X").reshape(K, 21, 10)[:, 1:, :3].astype(np.float64)
-        got = pl.debug("SAMPLE_DIST").reshape(K, 20).astype(np.float64)
+        x = pl.debug("SAMPLE_X").reshape(D, 21, 10)[:, 1:, :3].astype(np.float64)
+        got = pl.debug("SAMPLE_DIST").reshape(D, 20).astype(np.float64)
     finally:
         pl.close()
-    for s in range(0, K, 64):
+    for s in range(0, D, 64):
         want = np.sqrt(((x[s:s + 64, :, None] - p.astype(np.float64)) ** 2).sum(-1)).min(-1)
         g, near = got[s:s + 64], want < P["d_max"]
         edge = np.abs(want - P["d_max"]) < 1e-6
