@@ -572,8 +572,8 @@ __device__ __forceinline__ void rk4_vjp_stages(const float* x, const float* t2, 
 // Gradient refinement by a whole CTA (the update kernels): the forward
 // states by scans over the steps (rollout_by_scans); the backward pass split
 // by dependence (suffix sums for the position and velocity adjoints, the 4x4
-// attitude recurrence on one thread, the vector-Jacobian products of every
-// step in parallel); everything else over the CTA: the stage states of every
+// attitude recurrence as a scan of affine maps over four warps, the vector-Jacobian
+// products of every step in parallel); everything else over the CTA: the stage states of every
 // step, the nearest point of every
 // state (candidate lists cut into items of kRefItem entries; a 64-bit atomic
 // minimum of (squared distance bits, item index) keeps the lowest item among
@@ -701,8 +701,8 @@ __device__ void block_refine(float4* u, const float* guide, int T, const float* 
     // J^T (Lp, 0, Lv) (the step's vector-Jacobian product, in parallel), A the
     // 4x4 attitude Jacobian, whose transpose is applied in closed form: the
     // unnormalised y = q (x) m, so A^T l = ((l - yh (yh . l)) / |y|) (x) conj(m),
-    // yh = y / |y|; one thread chains it.  Then every step's dS/du_k is the
-    // control part of J_k^T L_{k+1}, in parallel.
+    // yh = y / |y|; its affine maps are composed by a scan.  Then every step's dS/du_k
+    // is the control part of J_k^T L_{k+1}, in parallel.
     {
       const float h = dp.dt;
       // (a) the suffix sums, thread t taking step k = T - 1 - t
@@ -847,26 +847,7 @@ __device__ void block_refine(float4* u, const float* guide, int T, const float* 
     }
     __syncthreads();
     // control terms, then the clamped step
-    if (tid < T) {
-      const int t = tid;
-      float4 a = rs.g[t];
-      const float4 ut = u[t];
-      if (t <= T - 2) {
-        a.x += 2.0f * cp.Q_c * ut.x; a.y += 2.0f * cp.Q_c * ut.y;
-        a.z += 2.0f * cp.Q_c * ut.z; a.w += 2.0f * cp.Q_c * ut.w;
-      }
-      if (t >= 1 && t <= T - 2) {
-        const float4 b = u[t - 1];
-        a.x += 2.0f * cp.Q_cd * (ut.x - b.x); a.y += 2.0f * cp.Q_cd * (ut.y - b.y);
-        a.z += 2.0f * cp.Q_cd * (ut.z - b.z); a.w += 2.0f * cp.Q_cd * (ut.w - b.w);
-      }
-      if (t + 1 >= 1 && t + 1 <= T - 2) {
-        const float4 c = u[t + 1];
-        a.x -= 2.0f * cp.Q_cd * (c.x - ut.x); a.y -= 2.0f * cp.Q_cd * (c.y - ut.y);
-        a.z -= 2.0f * cp.Q_cd * (c.z - ut.z); a.w -= 2.0f * cp.Q_cd * (c.w - ut.w);
-      }
-      rs.g[t] = a;
-    }
+    if (tid < T) rs.g[tid] = control_terms_grad(rs.g[tid], u, tid, T, cp);
     __syncthreads();
     if (tid < T) {
       const float4 a = u[tid], d = rs.g[tid];
