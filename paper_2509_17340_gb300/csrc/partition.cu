@@ -788,13 +788,14 @@ __device__ __forceinline__ void probe_lists(const ProbeArgs& p, const GridGeom& 
 }
 
 // K2c: the scatter pass and, in the remaining blocks, the {start, count} of
-// every cell (which needs only the scan) and the list probe.  Every block first turns
-// the scan's tile totals into tile offsets in shared memory (at most kMaxTiles of
-// them); block 0 also stores them.
-__global__ void __launch_bounds__(256) k_grid_scatter(CandArgs ca, int scatter_blocks,
-                                                      int2* __restrict__ range, int ncells,
-                                                      const int* tile_sum, int* tile_off,
-                                                      int ntiles, ProbeArgs probe) {
+// every cell (which needs only the scan).  Every block first turns the scan's
+// tile totals into tile offsets in shared memory (at most kMaxTiles of them);
+// block 0 also stores them.  kProbe: the first blocks are the list probe's (a kernel of its
+// own: the probe's arguments and branches cost the steps without it 0.2 us).
+template <bool kProbe>
+__device__ __forceinline__ void grid_scatter(const CandArgs& ca, int scatter_blocks, int2* __restrict__ range,
+                                             int ncells, const int* tile_sum, int* tile_off, int ntiles,
+                                             const ProbeArgs* probe) {
   pdl_start();
   __shared__ int s_off[kMaxTiles + 1];
   __shared__ int s_warp[32];
@@ -816,21 +817,36 @@ __global__ void __launch_bounds__(256) k_grid_scatter(CandArgs ca, int scatter_b
   if (blockIdx.x == 0)
     for (int i = threadIdx.x; i <= ntiles; i += blockDim.x) tile_off[i] = s_off[i];
   // the probe's blocks first: theirs is the longest chain
-  if ((int)blockIdx.x < probe.blocks) {
-    extern __shared__ __align__(16) unsigned char probe_smem[];
-    probe_lists(probe, ca.grid, ca.local, s_off, blockIdx.x, *reinterpret_cast<ProbeSmem*>(probe_smem));
-    return;
+  if constexpr (kProbe) {
+    if (blockIdx.x < kProbeBlocks) {
+      extern __shared__ __align__(16) unsigned char probe_smem[];
+      probe_lists(*probe, ca.grid, ca.local, s_off, blockIdx.x, *reinterpret_cast<ProbeSmem*>(probe_smem));
+      return;
+    }
   }
-  const int b = (int)blockIdx.x - probe.blocks;
+  const int b = (int)blockIdx.x - (kProbe ? kProbeBlocks : 0);
   if (b < scatter_blocks) {
     CandArgs a = ca;
     a.tile_off = s_off;
     cand_pass<true>(a, b, scatter_blocks);
     return;
   }
-  const int nrb = (int)gridDim.x - probe.blocks - scatter_blocks;
+  const int nrb = (int)gridDim.x - (kProbe ? kProbeBlocks : 0) - scatter_blocks;
   for (int c = (b - scatter_blocks) * blockDim.x + threadIdx.x; c < ncells; c += nrb * blockDim.x)
     range_cell(ca.local, s_off, ca.grid.cap, range, c);
+}
+
+__global__ void __launch_bounds__(256) k_grid_scatter(CandArgs ca, int scatter_blocks, int2* __restrict__ range,
+                                                      int ncells, const int* tile_sum, int* tile_off,
+                                                      int ntiles) {
+  grid_scatter<false>(ca, scatter_blocks, range, ncells, tile_sum, tile_off, ntiles, nullptr);
+}
+
+__global__ void __launch_bounds__(256) k_grid_scatter_probe(CandArgs ca, int scatter_blocks,
+                                                            int2* __restrict__ range, int ncells,
+                                                            const int* tile_sum, int* tile_off, int ntiles,
+                                                            ProbeArgs probe) {
+  grid_scatter<true>(ca, scatter_blocks, range, ncells, tile_sum, tile_off, ntiles, &probe);
 }
 
 // ---------------------------------------------------------------------------
@@ -1344,9 +1360,11 @@ cudaError_t launch_grid_scatter(const CandArgs& ca, int2* range, int ncells, con
   const int sms = device_sms();
   const int scatter_blocks = ca.n_items > 0 ? blocks_for(ca.n_items * 32, 256, 4 * sms) : 0;
   const int range_blocks = blocks_for(ncells, 256, 2 * sms);
-  return launch_ks(k_grid_scatter, dim3(probe.blocks + scatter_blocks + range_blocks), dim3(256),
-                   probe.blocks > 0 ? sizeof(ProbeSmem) : 0, s, true, ca, scatter_blocks, range, ncells,
-                   tile_sum, tile_off, ntiles, probe);
+  if (probe.blocks == 0)
+    return launch_k(k_grid_scatter, dim3(scatter_blocks + range_blocks), dim3(256), s, true, ca,
+                    scatter_blocks, range, ncells, tile_sum, tile_off, ntiles);
+  return launch_ks(k_grid_scatter_probe, dim3(kProbeBlocks + scatter_blocks + range_blocks), dim3(256),
+                   sizeof(ProbeSmem), s, true, ca, scatter_blocks, range, ncells, tile_sum, tile_off, ntiles, probe);
 }
 
 cudaError_t launch_grid_prune(PruneArgs a, cudaStream_t s) {
