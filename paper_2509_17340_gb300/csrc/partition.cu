@@ -863,9 +863,11 @@ __global__ void __launch_bounds__(256) k_grid_scatter_probe(CandArgs ca, int sca
 //
 // A list of 10 to 500 entries keeps a quarter to a tenth of them (the others lie
 // beside and behind the nearest ones), and Stage I's time is in scanning the longest
-// list of each warp's queries: with every kept point (178,000) 2.99 -> 0.95 ms, large
-// clutter 344 -> 277 us, flight cycle (split pass) 136 -> 67, a dense map 108 -> 48,
-// 64 batched planners 1055 -> 823, for 318, 36, 50, 70 and 221 us of pruning.
+// list of each warp's queries: with every kept point (178,000) 2.99 -> 0.78 ms, large
+// clutter 344 -> 278 us, flight cycle (split pass) 136 -> 70, a dense map 108 -> 51,
+// 64 batched planners 1055 -> 822, for 336, 36, 48, 68 and 224 us of pruning (one scene
+// each).  A single planner's launch returns at once where the list probe finds that its
+// samples meet too few entries for that (prunes_lists).
 // ---------------------------------------------------------------------------
 constexpr int kPruneMin = 5;        // shorter lists stay whole
 constexpr int kPruneThreads = 256;
